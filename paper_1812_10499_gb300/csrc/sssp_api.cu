@@ -134,9 +134,11 @@ int build_loop(Context& c) {
     }
     if (e == cudaSuccess && c.tail_ctas) {
         cudaGraphNode_t n3;
-        kp.func = const_cast<void*>(tail_fn(c.multi, c.narrow, c.P.pcnt != nullptr));
+        const TailKernel tk = tail_kernel(c.multi, c.narrow, c.P);
+        kp.func = const_cast<void*>(tk.fn);
         kp.gridDim = dim3(c.tail_ctas);
-        kp.sharedMemBytes = (unsigned)solve_smem_bytes(c.narrow);
+        kp.blockDim = dim3(tk.threads);
+        kp.sharedMemBytes = (unsigned)tk.smem;
         e = cudaGraphAddKernelNode(&n3, body, &n2, 1, &kp);
         if (e == cudaSuccess) {
             cudaLaunchAttributeValue v{};
@@ -180,7 +182,7 @@ int build_loop(Context& c) {
 int profile_graph_schedule(Context& c, cudaStream_t st) {
     const void* fr = relax_fn(c.multi, c.narrow, c.P.pcnt != nullptr);
     const void* fc = cupdate_fn(c.multi, c.narrow, c.P.pcnt != nullptr);
-    const void* ft = tail_fn(c.multi, c.narrow, c.P.pcnt != nullptr);
+    const TailKernel tk = tail_kernel(c.multi, c.narrow, c.P);
     const size_t smr = relax_smem_bytes(c.narrow), smc = cupdate_smem_bytes(c.narrow);
     RoundParams P = c.P;
     P.cond = 0;
@@ -212,8 +214,8 @@ int profile_graph_schedule(Context& c, cudaStream_t st) {
     ccfg.gridDim = dim3(c.grid_cup);
     ccfg.dynamicSmemBytes = smc;
     tcfg.gridDim = dim3(c.tail_ctas);
-    tcfg.blockDim = dim3(kThreads);
-    tcfg.dynamicSmemBytes = solve_smem_bytes(c.narrow);
+    tcfg.blockDim = dim3(tk.threads);
+    tcfg.dynamicSmemBytes = tk.smem;
     tcfg.stream = st;
     tcfg.attrs = at + 1 - nwin;
     tcfg.numAttrs = 1 + nwin;
@@ -233,7 +235,7 @@ int profile_graph_schedule(Context& c, cudaStream_t st) {
         CK(cudaEventRecord(c.ev[2], st));
         CK(cudaMemcpyAsync(&c.h_snap[0], c.P.ctl, sizeof(Ctl), cudaMemcpyDeviceToHost, st));
         CK(cudaEventRecord(c.ev[3], st));
-        CK(cudaLaunchKernelExC(&tcfg, ft, args));
+        CK(cudaLaunchKernelExC(&tcfg, tk.fn, args));
         CK(cudaEventRecord(c.ev[4], st));
         CK(cudaMemcpyAsync(&c.h_snap[1], c.P.ctl, sizeof(Ctl), cudaMemcpyDeviceToHost, st));
         CK(cudaStreamSynchronize(st));
@@ -474,6 +476,7 @@ int init_single_context(sssp_graph* h) {
     c.tail_ctas = h->tail_ctas;
     RoundParams& P = c.P;
     P.tail_items = h->tail_items;
+    P.small = h->n <= 0x7FFFFFFFu && h->m <= 0xFFFFFFFFull;
     P.g.out_off = h->out_off;
     P.g.out_adj = h->out_adj;
     P.g.in_off = h->in_off;

@@ -19,7 +19,15 @@ namespace sssp {
 const void* relax_fn(bool multi, bool narrow, bool pred);
 const void* cupdate_fn(bool multi, bool narrow, bool pred);
 const void* solve_fn(bool multi, bool narrow, bool pred);
-const void* tail_fn(bool multi, bool narrow, bool pred);
+// The cluster kernel of the small rounds: k_small for a single query's
+// label-setting or windowed rounds, else k_tail.
+struct TailKernel {
+    const void* fn;
+    u32 threads;
+    size_t smem;
+};
+TailKernel small_kernel(bool narrow, bool win);
+TailKernel tail_kernel(bool multi, bool narrow, const RoundParams& P);
 const void* barrier_selftest_fn();
 u32 tail_cluster_ctas();
 size_t solve_smem_bytes(bool narrow);

@@ -3,6 +3,7 @@
 // self-test, with the engine's access to them (kernel addresses, shared
 // memory, occupancy, start launches).  The kernels with SP_1's predecessor
 // counts come from sssp_round_pred.cu.
+#include "sssp_engine.h"
 #include "sssp_round.cuh"
 
 namespace sssp {
@@ -30,8 +31,15 @@ const void* cupdate_fn(bool multi, bool narrow, bool pred) {
 const void* solve_fn(bool multi, bool narrow, bool pred) {
     return kernel_of(RoundKernel::kSolve, multi, narrow, pred);
 }
-const void* tail_fn(bool multi, bool narrow, bool pred) {
-    return kernel_of(RoundKernel::kTail, multi, narrow, pred);
+namespace {
+TailKernel list_tail(bool multi, bool narrow, bool pred) {
+    return TailKernel{kernel_of(RoundKernel::kTail, multi, narrow, pred), 256,
+                      solve_smem_bytes(narrow)};
+}
+}  // namespace
+TailKernel tail_kernel(bool multi, bool narrow, const RoundParams& P) {
+    if (!multi && P.small && !P.pcnt && !P.lc) return small_kernel(narrow, P.win != 0);
+    return list_tail(multi, narrow, P.pcnt != nullptr);
 }
 const void* barrier_selftest_fn() { return (const void*)k_barrier_selftest; }
 
@@ -60,8 +68,17 @@ cudaError_t launch_start(bool multi, bool narrow, const RoundParams& P, u32 firs
 }
 
 namespace {
-// Raises the dynamic shared-memory limit of the four round kernels of one
-// family (default or counting) and allows the tail kernel's 16-CTA cluster.
+// Shared-memory limit and 16-CTA cluster of one tail kernel.
+cudaError_t set_tail_attributes(const TailKernel& k) {
+    cudaError_t e = cudaFuncSetAttribute(k.fn, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         (int)k.smem);
+    if (e == cudaSuccess)
+        e = cudaFuncSetAttribute(k.fn, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+    return e;
+}
+
+// Raises the dynamic shared-memory limit of the round kernels of one family
+// (default or counting) and allows the tail kernels' 16-CTA cluster.
 cudaError_t set_attributes(bool pred) {
     cudaError_t e = cudaSuccess;
     for (int v = 0; v < 4 && e == cudaSuccess; ++v) {
@@ -77,13 +94,8 @@ cudaError_t set_attributes(bool pred) {
             e = cudaFuncSetAttribute(solve_fn(multi, narrow, pred),
                                      cudaFuncAttributeMaxDynamicSharedMemorySize,
                                      (int)solve_smem_bytes(narrow));
-        if (e == cudaSuccess)
-            e = cudaFuncSetAttribute(tail_fn(multi, narrow, pred),
-                                     cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                     (int)solve_smem_bytes(narrow));
-        if (e == cudaSuccess)
-            e = cudaFuncSetAttribute(tail_fn(multi, narrow, pred),
-                                     cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+        if (e == cudaSuccess) e = set_tail_attributes(list_tail(multi, narrow, pred));
+        if (e == cudaSuccess && !pred) e = set_tail_attributes(small_kernel(narrow, multi));
     }
     return e;
 }
@@ -99,7 +111,7 @@ int blocks_per_sm(RoundKernel k, bool multi, bool narrow, bool pred, int threads
     return a;
 }
 
-int clusters_per_gpu(bool multi, bool narrow, bool pred) {
+int clusters_per_gpu(const TailKernel& k) {
     cudaLaunchConfig_t cfg = {};
     cudaLaunchAttribute at[1];
     at[0].id = cudaLaunchAttributeClusterDimension;
@@ -107,12 +119,12 @@ int clusters_per_gpu(bool multi, bool narrow, bool pred) {
     at[0].val.clusterDim.y = 1;
     at[0].val.clusterDim.z = 1;
     cfg.gridDim = dim3(kTailCTAs);
-    cfg.blockDim = dim3(256);
-    cfg.dynamicSmemBytes = solve_smem_bytes(narrow);
+    cfg.blockDim = dim3(k.threads);
+    cfg.dynamicSmemBytes = k.smem;
     cfg.attrs = at;
     cfg.numAttrs = 1;
     int n = 0;
-    if (cudaOccupancyMaxActiveClusters(&n, tail_fn(multi, narrow, pred), &cfg) != cudaSuccess) {
+    if (cudaOccupancyMaxActiveClusters(&n, k.fn, &cfg) != cudaSuccess) {
         (void)cudaGetLastError();
         return 0;
     }
@@ -143,7 +155,8 @@ cudaError_t pred_kernels_init() {
             if (blocks_per_sm(ks[i], multi, narrow, true, 256, sm[i]) <
                 blocks_per_sm(ks[i], multi, narrow, false, 256, sm[i]))
                 return cudaErrorInvalidConfiguration;
-        if (clusters_per_gpu(multi, narrow, true) < clusters_per_gpu(multi, narrow, false))
+        if (clusters_per_gpu(list_tail(multi, narrow, true)) <
+            clusters_per_gpu(list_tail(multi, narrow, false)))
             return cudaErrorInvalidConfiguration;
     }
     return cudaSuccess;
@@ -154,7 +167,9 @@ cudaError_t pred_kernels_init() {
 u32 tail_cluster_ctas() {
     if (round_kernels_init() != cudaSuccess) return 0;
     for (int v = 0; v < 4; ++v)
-        if (clusters_per_gpu(v & 1, (v >> 1) & 1, false) < 1) return 0;
+        if (clusters_per_gpu(list_tail(v & 1, (v >> 1) & 1, false)) < 1 ||
+            clusters_per_gpu(small_kernel(v & 1, (v >> 1) & 1)) < 1)
+            return 0;
     return kTailCTAs;
 }
 

@@ -1,0 +1,82 @@
+"""The cluster kernel of the small rounds against the oracle, at the sizes where
+its lists, its three ways of reading an entry's edges and its hand-over change."""
+import numpy as np
+import pytest
+
+import graphgen as gg
+import oracle
+from tests.test_gpu_parity import LAYOUTS, assert_parity
+
+pytestmark = pytest.mark.gpu
+
+
+def tree(fan, depth_weights, seed):
+    """Levels of fan[i] children per vertex, below a path of three vertices, with
+    an edge from every leaf's parent to a common sink."""
+    edges = [(0, 1, 5), (1, 2, 5), (2, 3, 5)]
+    level, n = [3], 4
+    for f, w in zip(fan, depth_weights):
+        nxt = []
+        for u in level:
+            ws = gg.uniform(seed, n, f, 1, w)
+            edges += [(u, n + i, int(ws[i])) for i in range(f)]
+            nxt += range(n, n + f)
+            n += f
+        level = nxt
+    sink = n
+    step = max(1, len(level) // 700)
+    edges += [(u, sink, 3) for u in level[::step]]
+    return gg.from_edges(n + 1, edges)
+
+
+def layers(sizes, wmax, seed):
+    """Layers of the given sizes, each fully linked to the next, behind a path."""
+    sizes = [1, 1] + list(sizes)
+    start = np.concatenate([[0], np.cumsum(sizes)])
+    n = int(start[-1])
+    deg = np.zeros(n, dtype=np.int64)
+    cols = []
+    for i in range(len(sizes) - 1):
+        deg[start[i]:start[i + 1]] = sizes[i + 1]
+        cols.append(np.tile(np.arange(start[i + 1], start[i + 2], dtype=np.uint32), sizes[i]))
+    col = np.concatenate(cols)
+    row_ptr = np.concatenate([[0], np.cumsum(deg)]).astype(np.uint64)
+    return gg.Graph(n, row_ptr, col, gg.uniform(seed, 1, len(col), 1, wmax).astype(np.uint32))
+
+
+MODES = pytest.mark.parametrize("mode,delta", [(oracle.RULE_THR, None), (oracle.RULE_MIND, None),
+                                               (oracle.CHEAP_FIRST, None), (oracle.RULE_THR, 7)],
+                                ids=["threshold", "mind", "cheap", "windowed"])
+
+
+@LAYOUTS
+@MODES
+@pytest.mark.parametrize("fan", [(3, 5), (100, 300), (40, 33, 17), (1, 1, 1500)],
+                         ids=["tiny", "overflow", "groups", "star"])
+def test_lists_grow_and_overflow(sssp_lib, layout, mode, delta, fan):
+    """Lists from a handful of entries to more than the cluster holds."""
+    assert_parity(sssp_lib, tree(fan, [50, 9, 1000], 11), 0, mode=mode, delta=delta, layout=layout)
+
+
+@LAYOUTS
+@MODES
+@pytest.mark.parametrize("sizes,hub", [((15,) * 6, 0), ((33,) * 6, 0), ((130,) * 4, 0),
+                                       ((520, 520), 0), ((520, 1200, 3), 1 << 20)],
+                         ids=["group", "row", "rows", "hub", "cta"])
+def test_entries_read_by_group_warp_and_cta(sssp_lib, layout, mode, delta, sizes, hub):
+    """Degrees on both sides of the limits between lanes, warp and CTA; the last
+    has more large entries than a CTA's list of them holds."""
+    opt = {"hub_degree": hub, "chunk_edges": 1024} if hub else {}
+    assert_parity(sssp_lib, layers(sizes, 40, len(sizes)), 0, mode=mode, delta=delta,
+                  layout=layout, **opt)
+
+
+@LAYOUTS
+@pytest.mark.parametrize("tail_items", ["1", "2", "40"])
+def test_hand_over_between_the_kernels(sssp_lib, layout, tail_items, monkeypatch):
+    """Rounds that cross the size limit in both directions, at both hand-over
+    points (after the relaxation, and at the end of a round)."""
+    monkeypatch.setenv("SSSP_TAIL_ITEMS", tail_items)
+    for g, s in ((gg.grid(60, 45, 1, 300, 3), 7), (gg.random_graph(3000, 5, 1, 60, 4), 1)):
+        assert_parity(sssp_lib, g, s, layout=layout)
+        assert_parity(sssp_lib, g, s, delta=20, layout=layout)
