@@ -369,6 +369,29 @@ __device__ __forceinline__ u32 static_item(u32 wib) {
     return wib * gridDim.x + rank;
 }
 
+// How a phase's lists are cut into work items.  A warp works through its item
+// batch by batch, and each batch waits for the one before; so when the lists
+// are too short to give every warp of the grid a full item, the items are made
+// smaller instead: list tiles of 2^ts entries (32 at most), hub chunks in 2^ps
+// parts of at least 128 edges.
+struct Split {
+    u32 ts, ps;
+    u32 tiles, parts;       // items of either kind
+};
+__device__ __forceinline__ Split split_work(const RoundParams& P, u32 entries, u32 chunks,
+                                            u32 nwarps) {
+    Split w;
+    w.ps = 0;
+    while (w.ps < 3 && (chunks << (w.ps + 1)) <= nwarps / 2 && (P.chunk >> (w.ps + 1)) >= 128)
+        ++w.ps;
+    w.parts = chunks << w.ps;
+    const u32 room = w.parts < nwarps / 2 ? nwarps - w.parts : nwarps / 2;
+    w.ts = 5;
+    while (w.ts > 0 && ((entries + (1u << (w.ts - 1)) - 1) >> (w.ts - 1)) <= room) --w.ts;
+    w.tiles = (entries + (1u << w.ts) - 1) >> w.ts;
+    return w;
+}
+
 // Accumulators a thread carries through one phase.
 struct Acc {
     u64 fmin_d, fmin_t;     // folds of minD / threshold (single-query mode)
@@ -759,15 +782,15 @@ __device__ __forceinline__ void relax_consume(const RoundParams& P, u32 cur, Acc
 
 template <bool MULTI, class L>
 __device__ void relax_small(const RoundParams& P, WarpStage<typename L::RSlot>& st, u32 t,
-                            u32 nfs, u32 cur, u32 lane, Acc& a, WarpQueue& q, WarpQueue& qf,
-                            Pend& pd, bool has_pre, u32 gpre) {
-    const u32 idx = t * 32 + lane;
-    const bool valid = idx < nfs;
+                            u32 ts, u32 nfs, u32 cur, u32 lane, Acc& a, WarpQueue& q,
+                            WarpQueue& qf, Pend& pd) {
+    const u32 idx = (t << ts) + lane;
+    const bool valid = (lane >> ts) == 0 && idx < nfs;
     u32 g = 0, xloc = 0, inst = 0, deg = 0;
     u64 gbase = 0, b = 0, dx = 0;
     const uint2* adj = P.g.out_adj;
     if (valid) {
-        g = has_pre ? gpre : P.L.FS[cur][idx];
+        g = P.L.FS[cur][idx];
         const InstDesc& d = desc_of<MULTI>(P, g, inst);
         gbase = d.base;
         adj = d.out_adj;
@@ -797,20 +820,22 @@ __device__ void relax_small(const RoundParams& P, WarpStage<typename L::RSlot>& 
 }
 
 template <bool MULTI, class L>
-__device__ void relax_hub(const RoundParams& P, WarpStage<typename L::RSlot>& st, u32 c, u32 nfh,
-                          u32 cur, u32 lane, Acc& a, WarpQueue& q, WarpQueue& qf, Pend& pd) {
+__device__ void relax_hub(const RoundParams& P, WarpStage<typename L::RSlot>& st, u32 item, u32 ps,
+                          u32 nfh, u32 cur, u32 lane, Acc& a, WarpQueue& q, WarpQueue& qf,
+                          Pend& pd) {
     const uint2* FH = P.L.FH[cur];
+    const u32 c = item >> ps, part = item & ((1u << ps) - 1u);
     const uint2 ent = FH[hub_entry(P, FH, P.L.FC[cur], nfh, c)];
     const u32 g = ent.x, k = c - ent.y;
     u32 inst;
     const InstDesc& d = desc_of<MULTI>(P, g, inst);
     const u32 xloc = g - (u32)d.base;
     const u64 b = d.out_off[xloc], e_end = d.out_off[xloc + 1];
-    const u64 cb = b + (u64)k * P.chunk;
-    const u64 ce = umin64(cb + P.chunk, e_end);
+    const u64 cb = b + (u64)k * P.chunk + ((P.chunk * part) >> ps);
+    const u64 ce = umin64(b + (u64)k * P.chunk + ((P.chunk * (part + 1)) >> ps), e_end);
     typename L::Rec* rx = L::rec(P) + g;
     const u64 dx = (P.lc || P.win) ? P.snap[g] : (L::ld_dc(rx, cur).y & kCMask);
-    if (k == 0 && lane == 0) {
+    if (k == 0 && part == 0 && lane == 0) {
         rx->cf[cur ^ 1] = rx->cf[cur];
         a.visits++;
     }
@@ -847,11 +872,6 @@ __device__ void relax_phase(const RoundParams& P, unsigned char* s_dyn, u32 r) {
     Ctl* ctl = P.ctl;
     const u32 cur = r & 1u, nxt = cur ^ 1u;
     const u32 lane = threadIdx.x & 31u, wib = threadIdx.x >> 5;
-    // The static item's small-list entry, loaded beside the list counts (one
-    // memory round trip fewer); it is used only if the item is a small tile.
-    const u32 item0 = static_item(wib);
-    const u32 pidx = item0 * 32 + lane;
-    const u32 gpre = pidx < P.L.capS ? P.L.FS[cur][pidx] : 0u;
 
     if (blockIdx.x == 0) {
         // Open the slots of round r + 1 (last read in round r - 1).
@@ -883,11 +903,12 @@ __device__ void relax_phase(const RoundParams& P, unsigned char* s_dyn, u32 r) {
     const u32 nfs = min(ctl->nFS[cur], P.L.capS);
     const u64 fhpk = ctl->FHpk[cur];
     const u32 nfh = min((u32)(fhpk >> 32), P.L.capH), fh_chunks = (u32)fhpk;
-    const u32 tiles = (nfs + 31) >> 5;
+    const u32 nwarps = gridDim.x * kWarps;
+    const Split w = split_work(P, nfs, fh_chunks, nwarps);
     // Label-correcting and windowed: copy the fixed lower-bound word of the
     // vertices fixed last round into the other parity slot (32 per item).
     const u32 nfx = (P.lc || P.win) ? min(ctl->nFX[cur], P.L.capS) : 0u;
-    const u32 total = tiles + fh_chunks + ((nfx + 31) >> 5);
+    const u32 total = w.tiles + w.parts + ((nfx + 31) >> 5);
 
     Acc a = {kInf64, kInf64, 0, 0, 0};
     WarpQueue q = {s_q + wib * kQCap, 0};
@@ -896,15 +917,13 @@ __device__ void relax_phase(const RoundParams& P, unsigned char* s_dyn, u32 r) {
     pd.any = false;
     pd.r = r;
     // First item per warp is static (no atomic); the rest are pulled.
-    const u32 nwarps = gridDim.x * kWarps;
-    for (u32 item = item0; item < total;) {
-        if (item < tiles) {
-            relax_small<MULTI, L>(P, s_st[wib], item, nfs, cur, lane, a, q, qf, pd,
-                                  item == item0, gpre);
-        } else if (item < tiles + fh_chunks) {
-            relax_hub<MULTI, L>(P, s_st[wib], item - tiles, nfh, cur, lane, a, q, qf, pd);
+    for (u32 item = static_item(wib); item < total;) {
+        if (item < w.tiles) {
+            relax_small<MULTI, L>(P, s_st[wib], item, w.ts, nfs, cur, lane, a, q, qf, pd);
+        } else if (item < w.tiles + w.parts) {
+            relax_hub<MULTI, L>(P, s_st[wib], item - w.tiles, w.ps, nfh, cur, lane, a, q, qf, pd);
         } else {
-            const u32 idx = (item - tiles - fh_chunks) * 32 + lane;
+            const u32 idx = (item - w.tiles - w.parts) * 32 + lane;
             if (idx < nfx) {
                 typename L::Rec* rx = L::rec(P) + P.L.FX[cur][idx];
                 rx->cf[nxt] = rx->cf[cur];
@@ -978,19 +997,19 @@ __device__ __forceinline__ u64 decide(const RoundParams& P, u64 dy, u64 cy, u64 
 // faster, and with the wide layout's 64-bit terms the atomics cost 1.4% on
 // the 4096^2 grid, so both keep the scan.
 template <bool MULTI, class L, bool SHATOM = false>
-__device__ void cup_small(const RoundParams& P, WarpStage<typename L::CSlot>& st, u32 t, u32 nas,
-                          u32 r, u32 cur, u32 lane, u64* smin, u64 thr0, u64 minD0, Acc& a,
-                          Acc& an, WarpQueue& qf, WarpQueue& qa, bool has_pre, u32 gpre) {
+__device__ void cup_small(const RoundParams& P, WarpStage<typename L::CSlot>& st, u32 t, u32 ts,
+                          u32 nas, u32 r, u32 cur, u32 lane, u64* smin, u64 thr0, u64 minD0,
+                          Acc& a, Acc& an, WarpQueue& qf, WarpQueue& qa) {
     const u32 nxt = cur ^ 1u;
-    const u32 idx = t * 32 + lane;
-    const bool valid = idx < nas;
+    const u32 idx = (t << ts) + lane;
+    const bool valid = (lane >> ts) == 0 && idx < nas;
     u32 g = 0, yloc = 0, inst = 0, deg = 0, outw = kNoOutW;
     u64 gbase = 0, ib = 0, dy = 0, cy = 0, thr = thr0, minD = minD0, odeg = 0;
     bool fix_now = false;
     const uint2* in_adj = P.g.in_adj;
     typename L::Rec* rec = L::rec(P);
     if (valid) {
-        g = has_pre ? gpre : P.L.AS[cur][idx];
+        g = P.L.AS[cur][idx];
         const InstDesc& d = desc_of<MULTI>(P, g, inst);
         gbase = d.base;
         in_adj = d.in_adj;
@@ -1105,9 +1124,10 @@ __device__ void cup_small(const RoundParams& P, WarpStage<typename L::CSlot>& st
 }
 
 template <bool MULTI, class L>
-__device__ void cup_hub(const RoundParams& P, WarpStage<typename L::CSlot>& st, u32 c, u32 nah,
-                        u32 r, u32 cur, u32 lane, u64 thr0, u64 minD0, Acc& a, Acc& an) {
+__device__ void cup_hub(const RoundParams& P, WarpStage<typename L::CSlot>& st, u32 item, u32 ps,
+                        u32 nah, u32 r, u32 cur, u32 lane, u64 thr0, u64 minD0, Acc& a, Acc& an) {
     const u32 nxt = cur ^ 1u;
+    const u32 c = item >> ps, part = item & ((1u << ps) - 1u);
     const uint2* AH = P.L.AH[cur];
     const u32 lo = hub_entry(P, AH, P.L.AC[cur], nah, c);
     const uint2 ent = AH[lo];
@@ -1122,8 +1142,8 @@ __device__ void cup_hub(const RoundParams& P, WarpStage<typename L::CSlot>& st, 
     const u32 yloc = g - (u32)d.base;
     const u64 ib = d.in_off[yloc], ie = d.in_off[yloc + 1];
     const u32 nch = (u32)((ie - ib + P.chunk - 1) / P.chunk);   // as counted by put_hub
-    const u64 cb = ib + (u64)k * P.chunk;
-    const u64 ce = umin64(cb + P.chunk, ie);
+    const u64 cb = ib + (u64)k * P.chunk + ((P.chunk * part) >> ps);
+    const u64 ce = umin64(ib + (u64)k * P.chunk + ((P.chunk * (part + 1)) >> ps), ie);
     const typename L::Bounds bd = L::bounds(thr, minD);
     typename L::Term tv = L::kTermInf;
     // Cheaper rules first: every chunk of y takes the same decision (the
@@ -1160,8 +1180,8 @@ __device__ void cup_hub(const RoundParams& P, WarpStage<typename L::CSlot>& st, 
                  : "=r"(arrived)
                  : "l"(&P.L.hubcnt[lo])
                  : "memory");
-    if (arrived != nch - 1) return;
-    // Last chunk of this hub: finish the vertex.
+    if (arrived != (nch << ps) - 1) return;
+    // Last part of this hub's last chunk: finish the vertex.
     const u64 m = atomicExch(&P.L.hubmin[lo], kInf64);
     P.L.hubcnt[lo] = 0;
     typename L::Rec* ry = L::rec(P) + g;
@@ -1290,11 +1310,6 @@ __device__ void cupdate_phase(const RoundParams& P, unsigned char* s_dyn, u32 r)
     Ctl* ctl = P.ctl;
     const u32 cur = r & 1u, nxt = cur ^ 1u;
     const u32 lane = threadIdx.x & 31u, wib = threadIdx.x >> 5;
-    // The static item's small-list entry, loaded beside the list counts (as
-    // in relax_phase).
-    const u32 item0 = static_item(wib);
-    const u32 pidx = item0 * 32 + lane;
-    const u32 gpre = pidx < P.L.capS ? P.L.AS[cur][pidx] : 0u;
     if (blockIdx.x == 0 && threadIdx.x == 0) ctl->work[0] = 0;
     if (P.lc && blockIdx.x == 0) {
         // Label-correcting: the next relaxation appends the frontier after it
@@ -1309,7 +1324,8 @@ __device__ void cupdate_phase(const RoundParams& P, unsigned char* s_dyn, u32 r)
     const u32 nas = min(ctl->nAS[cur], P.L.capS);
     const u64 ahpk = ctl->AHpk[cur];
     const u32 nah = min((u32)(ahpk >> 32), P.L.capH), ah_chunks = (u32)ahpk;
-    const u32 tiles = (nas + 31) >> 5;
+    const u32 nwarps = gridDim.x * kWarps;
+    const Split w = split_work(P, nas, ah_chunks, nwarps);
     // Label-correcting: also record the distance of every next-frontier
     // vertex while D is stable (its relaxation reads it next round).
     u32 sfs = 0, sfh = 0, snap_items = 0;
@@ -1318,7 +1334,7 @@ __device__ void cupdate_phase(const RoundParams& P, unsigned char* s_dyn, u32 r)
         sfh = min((u32)(ctl->FHpk[nxt] >> 32), P.L.capH);
         snap_items = ((sfs + 31) >> 5) + ((sfh + 31) >> 5);
     }
-    const u32 total = tiles + ah_chunks + snap_items;
+    const u32 total = w.tiles + w.parts + snap_items;
     u64 thr = kInf64, minD = kInf64;
     if (!MULTI) {
         thr = P.ivar[0].thr[cur];
@@ -1329,15 +1345,15 @@ __device__ void cupdate_phase(const RoundParams& P, unsigned char* s_dyn, u32 r)
     Acc an = {kInf64, kInf64, 0, 0, 0};
     WarpQueue qf = {s_qf + wib * kQCap, 0}, qa = {s_qa + wib * kQCap, 0};
     // First item per warp is static (no atomic); the rest are pulled.
-    const u32 nwarps = gridDim.x * kWarps;
-    for (u32 item = item0; item < total;) {
-        if (item < tiles)
-            cup_small<MULTI, L, TAIL>(P, s_st[wib], item, nas, r, cur, lane, s_min + wib * 32,
-                                      thr, minD, a, an, qf, qa, item == item0, gpre);
-        else if (item < tiles + ah_chunks)
-            cup_hub<MULTI, L>(P, s_st[wib], item - tiles, nah, r, cur, lane, thr, minD, a, an);
+    for (u32 item = static_item(wib); item < total;) {
+        if (item < w.tiles)
+            cup_small<MULTI, L, TAIL>(P, s_st[wib], item, w.ts, nas, r, cur, lane,
+                                      s_min + wib * 32, thr, minD, a, an, qf, qa);
+        else if (item < w.tiles + w.parts)
+            cup_hub<MULTI, L>(P, s_st[wib], item - w.tiles, w.ps, nah, r, cur, lane, thr, minD, a,
+                              an);
         else
-            snap_frontier<L>(P, item - tiles - ah_chunks, nxt, sfs, sfh, lane);
+            snap_frontier<L>(P, item - w.tiles - w.parts, nxt, sfs, sfh, lane);
         __syncwarp();
         if (total <= nwarps) break;                // the static items were all
         u32 next = 0;
