@@ -246,9 +246,9 @@ int profile_graph_schedule(Context& c, cudaStream_t st) {
         const Ctl& A = c.h_snap[0];
         const Ctl& B = c.h_snap[1];
         for (int i = 0; i < 4; ++i) {
-            c.prof_grid_ctr[i] += A.stats[i] - prev.stats[i];
-            c.prof_tail_ctr[i] += B.stats[i] - A.stats[i];
-            c.prof_round_ctr.push_back(A.stats[i] - prev.stats[i]);
+            c.prof_grid_ctr[i] += A.stats[i].v - prev.stats[i].v;
+            c.prof_tail_ctr[i] += B.stats[i].v - A.stats[i].v;
+            c.prof_round_ctr.push_back(A.stats[i].v - prev.stats[i].v);
         }
         const u32 tr = B.round - A.round;
         c.prof_relax_ms += a;
@@ -296,7 +296,7 @@ int run_loop(Context& c, u32 loop_mode, cudaStream_t st) {
             P.trace = c.trace;
             P.trace_cap = c.trace_cap;
             P.trace_base = c.h_ctl->round;
-            for (int i = 0; i < 4; ++i) c.prof_grid_ctr[i] -= c.h_ctl->stats[i];
+            for (int i = 0; i < 4; ++i) c.prof_grid_ctr[i] -= c.h_ctl->stats[i].v;
         }
         void* args[] = {&P};
         const void* fs = solve_fn(c.multi, c.narrow, c.P.pcnt != nullptr);
@@ -305,7 +305,7 @@ int run_loop(Context& c, u32 loop_mode, cudaStream_t st) {
         if (c.prof) {
             CK(cudaMemcpyAsync(c.h_ctl, c.P.ctl, sizeof(Ctl), cudaMemcpyDeviceToHost, st));
             CK(cudaStreamSynchronize(st));
-            for (int i = 0; i < 4; ++i) c.prof_grid_ctr[i] += c.h_ctl->stats[i];
+            for (int i = 0; i < 4; ++i) c.prof_grid_ctr[i] += c.h_ctl->stats[i].v;
             const u32 rounds = std::min<u32>(c.h_ctl->round - P.trace_base, (c.trace_cap - 1) / 2);
             std::vector<u64> t(2 * rounds + 1);
             CK(cudaMemcpy(t.data(), c.trace, sizeof(u64) * t.size(), cudaMemcpyDeviceToHost));
@@ -391,7 +391,7 @@ int run_loop(Context& c, u32 loop_mode, cudaStream_t st) {
         if (c.h_ctl->status != kRunning || c.h_ctl->round > c.h_ctl->stop_round) break;
     }
     if (c.prof)
-        for (int i = 0; i < 4; ++i) c.prof_grid_ctr[i] += c.h_ctl->stats[i] - start_ctl.stats[i];
+        for (int i = 0; i < 4; ++i) c.prof_grid_ctr[i] += c.h_ctl->stats[i].v - start_ctl.stats[i].v;
     return SSSP_OK;
 }
 
@@ -1240,11 +1240,11 @@ int sssp_solve_ex(sssp_handle h, uint32_t source, const sssp_solve_args* args,
     if (info) {
         info->rounds = v.rounds;
         info->finished = v.status == kDone;
-        info->out_scanned = c.h_ctl->stats[0];
-        info->in_scanned = c.h_ctl->stats[1];
-        info->active_visits = c.h_ctl->stats[2];
-        info->front_visits = c.h_ctl->stats[3];
-        info->reached = c.h_ctl->stats[4];
+        info->out_scanned = c.h_ctl->stats[0].v;
+        info->in_scanned = c.h_ctl->stats[1].v;
+        info->active_visits = c.h_ctl->stats[2].v;
+        info->front_visits = c.h_ctl->stats[3].v;
+        info->reached = c.h_ctl->stats[4].v;
         info->kernel_launches = 4 + c.launches_per_iter * (u64)c.h_ctl->body_iters +
                                 (c.last_loop == SSSP_LOOP_PERSISTENT ? 1 : 0);
     }

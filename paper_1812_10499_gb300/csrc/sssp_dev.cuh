@@ -75,20 +75,22 @@ struct __align__(16) InstVar {
 };
 constexpr u32 kNoTarget = 0xFFFFFFFFu;
 
-// Engine control block (one per solve context).
-struct __align__(16) Ctl {
+// Engine control block (one per solve context).  Words that every CTA of a
+// round kernel updates lie 128 bytes apart: atomics on one L2 slice are served
+// one by one, those on different slices side by side.
+struct __align__(128) HotWord {
+    u32 v;
+};
+struct __align__(128) HotCount {
+    u64 v;
+};
+struct __align__(128) Ctl {
     u32 round;          // next engine round to execute
     u32 status;         // kRunning while any query runs, kDone otherwise, kErrRounds
     u32 running;        // queries still running after the last round
     u32 stop_round;     // device loop stops after this round (serving steps)
     u32 round_limit;    // hard cap; exceeding it is an internal error
     u32 error;          // nonzero: a list capacity was exceeded (bug guard)
-    u32 nFS[2];         // frontier, small-degree entries
-    u32 nAS[2];         // active, small-degree entries
-    u64 FHpk[2];        // frontier hubs: (entries << 32) | chunks
-    u64 AHpk[2];        // active hubs: (entries << 32) | chunks
-    u32 work[2];        // dynamic work counters of the two round kernels
-    u32 done_ctas;      // arrival counter for the end-of-round epilogue
     u32 ninst;          // number of query slots
     u32 loop_iters;     // loop bodies started (watchdog against a stuck loop)
     u32 bar_count;      // grid barrier of the persistent kernel: arrivals
@@ -99,7 +101,13 @@ struct __align__(16) Ctl {
     u32 body_iters;     // launches of the relax kernel (one per loop iteration)
     u32 nFX[2];         // label-correcting: vertices fixed in the round (see Lists::FX)
 
-    u64 stats[5];       // out-edges scanned, in-edges scanned, active visits, frontier
+    __align__(128) u32 nFS[2];    // frontier, small-degree entries
+    __align__(128) u32 nAS[2];    // active, small-degree entries
+    __align__(128) u64 FHpk[2];   // frontier hubs: (entries << 32) | chunks
+    __align__(128) u64 AHpk[2];   // active hubs: (entries << 32) | chunks
+    HotWord work[2];              // dynamic work counters of the two round kernels
+    __align__(128) u32 done_ctas; // arrival counter for the end-of-round epilogue
+    HotCount stats[5];  // out-edges scanned, in-edges scanned, active visits, frontier
                         // visits, vertices fixed (single query)
 };
 

@@ -37,7 +37,8 @@ namespace sssp {
 constexpr u32 kFull = 0xFFFFFFFFu;
 constexpr u32 kWarps = 8;       // warps per CTA (256 threads)
 constexpr u32 kSmallGrid = 32;  // grids up to this many CTAs run latency-bound rounds
-constexpr u32 kQCap = 64;       // entries of a warp append buffer
+constexpr u32 kQFlush = 96;     // entries a warp append buffer hands over per atomic
+constexpr u32 kQCap = kQFlush + 32;
 // Build-time tuning: CTAs per SM the round kernels are compiled for, and
 // edges per warp batch of the copy pipeline.
 #ifndef SSSP_MIN_CTAS
@@ -292,8 +293,9 @@ __device__ __forceinline__ u32 hub_entry(const RoundParams& P, const uint2* list
     return lo;
 }
 
-// Warp-private append buffer of one small list (in shared memory); the
-// count is warp-uniform.  32 entries leave per global atomicAdd.
+// Warp-private append buffer of one small list (in shared memory); the count
+// is warp-uniform.  A full buffer leaves kQFlush entries per global atomic; what
+// is left at the end of a phase leaves with the CTA's other warps (end_phase).
 struct WarpQueue {
     u32* buf;
     u32 cnt;
@@ -306,46 +308,18 @@ __device__ __forceinline__ void wq_push(const RoundParams& P, WarpQueue& q, u32*
     if (pred) q.buf[q.cnt + __popc(mask & ((1u << lane) - 1u))] = g;
     q.cnt += __popc(mask);
     __syncwarp();
-    if (q.cnt >= 32) {
+    if (q.cnt >= kQFlush) {
         u32 base = 0;
-        if (lane == 0) base = atomicAdd(counter, 32u);
+        if (lane == 0) base = atomicAdd(counter, kQFlush);
         base = __shfl_sync(kFull, base, 0);
-        put_small(P, list, base + lane, q.buf[lane]);
-        const u32 rest = q.cnt - 32;
-        const u32 v = (lane < rest) ? q.buf[32 + lane] : 0u;
+#pragma unroll
+        for (u32 i = 0; i < kQFlush; i += 32) put_small(P, list, base + i + lane, q.buf[i + lane]);
+        q.cnt -= kQFlush;
+        const u32 v = (lane < q.cnt) ? q.buf[kQFlush + lane] : 0u;
         __syncwarp();
-        if (lane < rest) q.buf[lane] = v;
+        if (lane < q.cnt) q.buf[lane] = v;
         __syncwarp();
-        q.cnt = rest;
     }
-}
-
-__device__ __forceinline__ void wq_flush(const RoundParams& P, WarpQueue& q, u32* counter,
-                                         u32* list, u32 lane) {
-    if (q.cnt == 0) return;
-    u32 base = 0;
-    if (lane == 0) base = atomicAdd(counter, q.cnt);
-    base = __shfl_sync(kFull, base, 0);
-    if (lane < q.cnt) put_small(P, list, base + lane, q.buf[lane]);
-    __syncwarp();
-    q.cnt = 0;
-}
-
-// Flushes two queues; both counter atomics are in flight together.
-__device__ __forceinline__ void wq_flush2(const RoundParams& P, WarpQueue& q1, u32* c1, u32* l1,
-                                          WarpQueue& q2, u32* c2, u32* l2, u32 lane) {
-    u32 b1 = 0, b2 = 0;
-    if (lane == 0) {
-        if (q1.cnt) b1 = atomicAdd(c1, q1.cnt);
-        if (q2.cnt) b2 = atomicAdd(c2, q2.cnt);
-    }
-    b1 = __shfl_sync(kFull, b1, 0);
-    b2 = __shfl_sync(kFull, b2, 0);
-    if (lane < q1.cnt) put_small(P, l1, b1 + lane, q1.buf[lane]);
-    if (lane < q2.cnt) put_small(P, l2, b2 + lane, q2.buf[lane]);
-    __syncwarp();
-    q1.cnt = 0;
-    q2.cnt = 0;
 }
 
 // Appends g (where pred holds) to a small list with one atomic per warp.
@@ -392,6 +366,23 @@ __device__ __forceinline__ Split split_work(const RoundParams& P, u32 entries, u
     return w;
 }
 
+// The next work item of a warp: the rest of the run it took from the shared
+// counter last, or a new run.  A run is an eighth of the warp's even share of
+// what is left, so that a large phase makes few atomics on the counter and its
+// end is still dealt item by item.
+__device__ __forceinline__ u32 next_item(u32* counter, u32 item, u32& left, u32 total, u32 nwarps,
+                                         u32 lane) {
+    if (left) {
+        --left;
+        return item + 1;
+    }
+    const u32 run = min(8u, max(1u, (total - item) / (8u * nwarps)));
+    u32 first = 0;
+    if (lane == 0) first = atomicAdd(counter, run) + nwarps;
+    left = run - 1;
+    return __shfl_sync(kFull, first, 0);
+}
+
 // Accumulators a thread carries through one phase.
 struct Acc {
     u64 fmin_d, fmin_t;     // folds of minD / threshold (single-query mode)
@@ -416,53 +407,76 @@ __device__ __forceinline__ void fold(const RoundParams& P, u32 inst, u32 slot, u
     }
 }
 
-// Flush register folds and counters at the end of a phase (all lanes).
-template <bool MULTI, bool NARROW = false>
-__device__ __forceinline__ void flush(const RoundParams& P, u32 slot, u32 nfix_slot, Acc& a,
-                                      u32 lane, int stat_edges, int stat_visits) {
-    if (NARROW && gridDim.x <= kSmallGrid) {
-        // Cluster-sized grid, compact layout: every sum and minimum fits 32
-        // bits (distances below 2^31, D + outWeight below 2^32 - 2), so one
-        // warp reduction each instead of shuffle trees.
-        const u32 e32 = __reduce_add_sync(kFull, (u32)a.edges);
-        const u32 v32 = __reduce_add_sync(kFull, (u32)a.visits);
-        const u32 nf32 = __reduce_add_sync(kFull, (u32)a.nfix);
-        if (!MULTI) {
+// End of a phase: the warps' remaining list entries, folds and counters leave
+// together, with one atomic per word and CTA (all threads of the CTA).  The
+// words are shared by the whole grid, and an atomic on one word takes about 4
+// cycles of its L2 slice: one per warp, from 3648 warps, would take 7 us a word.
+template <bool MULTI, bool NARROW>
+__device__ __forceinline__ void end_phase(const RoundParams& P, u32 slot, u32 nfix_slot,
+                                          const Acc& a, u32 stat_edges, u32 stat_visits,
+                                          const WarpQueue& q0, u32* c0, u32* l0,
+                                          const WarpQueue& q1, u32* c1, u32* l1, u32 lane,
+                                          u32 wib) {
+    __shared__ u32 s_cnt[2][kWarps], s_base[2], s_nfix[kWarps], s_visits[kWarps];
+    __shared__ u64 s_mind[kWarps], s_mint[kWarps], s_edges[kWarps];
+    // (A warp's share of one phase's visits fits 32 bits.)
+    const u64 e = warp_sum64(a.edges);
+    const u32 v = __reduce_add_sync(kFull, (u32)a.visits);
+    u64 d = kInf64, t = kInf64;
+    u32 nf = 0;
+    if (!MULTI) {
+        if (NARROW) {
+            // Compact layout: distances below 2^31, D + outWeight below 2^32 - 2.
             const u32 d32 = __reduce_min_sync(kFull, a.fmin_d == kInf64 ? kFull : (u32)a.fmin_d);
             const u32 t32 = __reduce_min_sync(kFull, a.fmin_t == kInf64 ? kFull : (u32)a.fmin_t);
-            if (lane == 0) {
-                if (d32 != kFull) atomicMin(&P.ivar[0].minD[slot], (u64)d32);
-                if (t32 != kFull) atomicMin(&P.ivar[0].thr[slot], (u64)t32);
-                if (nf32) atomicAdd(&P.ivar[0].nfix[nfix_slot], nf32);
-            }
+            d = d32 == kFull ? kInf64 : d32;
+            t = t32 == kFull ? kInf64 : t32;
+        } else {
+            d = warp_min64(a.fmin_d);
+            t = warp_min64(a.fmin_t);
         }
-        if (lane == 0) {
-            if (e32) atomicAdd(&P.ctl->stats[stat_edges], (u64)e32);
-            if (v32) atomicAdd(&P.ctl->stats[stat_visits], (u64)v32);
-        }
-        return;
-    }
-    const u64 e = warp_sum64(a.edges), v = warp_sum64(a.visits);
-    const u64 nf = warp_sum64(a.nfix);
-    if (!MULTI) {
-        const u64 d = warp_min64(a.fmin_d), t = warp_min64(a.fmin_t);
-        if (lane == 0) {
-            // A large grid first reads the minimum, so that most warps skip
-            // the atomic on this one address; a cluster-sized grid (few
-            // warps, latency-bound rounds) fires the atomics without waiting.
-            if (gridDim.x > kSmallGrid) {
-                if (d != kInf64) atomic_min_checked(&P.ivar[0].minD[slot], d);
-                if (t != kInf64) atomic_min_checked(&P.ivar[0].thr[slot], t);
-            } else {
-                if (d != kInf64) atomicMin(&P.ivar[0].minD[slot], d);
-                if (t != kInf64) atomicMin(&P.ivar[0].thr[slot], t);
-            }
-            if (nf) atomicAdd(&P.ivar[0].nfix[nfix_slot], (u32)nf);
-        }
+        nf = __reduce_add_sync(kFull, a.nfix);
     }
     if (lane == 0) {
-        if (e) atomicAdd(&P.ctl->stats[stat_edges], e);
-        if (v) atomicAdd(&P.ctl->stats[stat_visits], v);
+        s_cnt[0][wib] = q0.cnt;
+        s_cnt[1][wib] = q1.cnt;
+        s_mind[wib] = d;
+        s_mint[wib] = t;
+        s_edges[wib] = e;
+        s_visits[wib] = v;
+        s_nfix[wib] = nf;
+    }
+    __syncthreads();
+    const bool in = lane < kWarps;
+    if (wib == 0) {
+        const u32 n0 = __reduce_add_sync(kFull, in ? s_cnt[0][lane] : 0u);
+        const u32 n1 = __reduce_add_sync(kFull, in ? s_cnt[1][lane] : 0u);
+        if (lane < 2) {
+            const u32 n = lane ? n1 : n0;
+            u32 base = 0;
+            if (n) base = atomicAdd(lane ? c1 : c0, n);
+            s_base[lane] = base;
+        }
+    } else if (wib == 1) {
+        const u64 et = warp_sum64(in ? s_edges[lane] : 0ull);
+        const u32 vt = __reduce_add_sync(kFull, in ? s_visits[lane] : 0u);
+        if (lane == 0 && et) atomicAdd(&P.ctl->stats[stat_edges].v, et);
+        if (lane == 0 && vt) atomicAdd(&P.ctl->stats[stat_visits].v, (u64)vt);
+    } else if (!MULTI && wib == 2) {
+        const u64 dm = warp_min64(in ? s_mind[lane] : kInf64);
+        const u64 tm = warp_min64(in ? s_mint[lane] : kInf64);
+        const u32 nft = __reduce_add_sync(kFull, in ? s_nfix[lane] : 0u);
+        if (lane == 0 && dm != kInf64) atomicMin(&P.ivar[0].minD[slot], dm);
+        if (lane == 0 && tm != kInf64) atomicMin(&P.ivar[0].thr[slot], tm);
+        if (lane == 0 && nft) atomicAdd(&P.ivar[0].nfix[nfix_slot], nft);
+    }
+    __syncthreads();
+#pragma unroll
+    for (u32 k = 0; k < 2; ++k) {
+        const WarpQueue& q = k ? q1 : q0;
+        u32 base = s_base[k];
+        for (u32 w = 0; w < wib; ++w) base += s_cnt[k][w];
+        for (u32 i = lane; i < q.cnt; i += 32) put_small(P, k ? l1 : l0, base + i, q.buf[i]);
     }
 }
 
@@ -888,7 +902,7 @@ __device__ void relax_phase(const RoundParams& P, unsigned char* s_dyn, u32 r) {
             ctl->nAS[nxt] = 0;
             ctl->AHpk[nxt] = 0;
             ctl->nFX[nxt] = 0;
-            ctl->work[1] = 0;
+            ctl->work[1].v = 0;
             ctl->done_ctas = 0;
         }
         for (u32 i = threadIdx.x; i < ctl->ninst; i += blockDim.x) {
@@ -917,6 +931,7 @@ __device__ void relax_phase(const RoundParams& P, unsigned char* s_dyn, u32 r) {
     pd.any = false;
     pd.r = r;
     // First item per warp is static (no atomic); the rest are pulled.
+    u32 left = 0;
     for (u32 item = static_item(wib); item < total;) {
         if (item < w.tiles) {
             relax_small<MULTI, L>(P, s_st[wib], item, w.ts, nfs, cur, lane, a, q, qf, pd);
@@ -930,13 +945,11 @@ __device__ void relax_phase(const RoundParams& P, unsigned char* s_dyn, u32 r) {
             }
         }
         if (total <= nwarps) break;                // the static items were all
-        u32 next = 0;
-        if (lane == 0) next = atomicAdd(&ctl->work[0], 1u) + nwarps;
-        item = __shfl_sync(kFull, next, 0);
+        item = next_item(&ctl->work[0].v, item, left, total, nwarps, lane);
     }
     relax_consume<MULTI, L>(P, cur, a, q, qf, pd, lane);
-    wq_flush2(P, q, &ctl->nAS[cur], P.L.AS[cur], qf, &ctl->nFS[nxt], P.L.FS[nxt], lane);
-    flush<MULTI, L::kNarrow>(P, cur, nxt, a, lane, 0, 3);
+    end_phase<MULTI, L::kNarrow>(P, cur, nxt, a, 0, 3, q, &ctl->nAS[cur], P.L.AS[cur], qf,
+                                 &ctl->nFS[nxt], P.L.FS[nxt], lane, wib);
 }
 
 template <bool MULTI, class L>
@@ -1264,7 +1277,7 @@ __device__ inline void round_epilogue(const RoundParams& P, u32 r) {
         const u32 total = s_running;
         // Vertices fixed this round (single query): label-setting counts them
         // in nfix, label-correcting and windowed relaxation list them in FX.
-        if (ninst == 1) ctl->stats[4] += (P.lc || P.win) ? ctl->nFX[nxt] : P.ivar[0].nfix[nxt];
+        if (ninst == 1) ctl->stats[4].v += (P.lc || P.win) ? ctl->nFX[nxt] : P.ivar[0].nfix[nxt];
         ctl->running = total;
         ctl->cup_only = 0;
         ctl->round = r + 1;
@@ -1310,7 +1323,7 @@ __device__ void cupdate_phase(const RoundParams& P, unsigned char* s_dyn, u32 r)
     Ctl* ctl = P.ctl;
     const u32 cur = r & 1u, nxt = cur ^ 1u;
     const u32 lane = threadIdx.x & 31u, wib = threadIdx.x >> 5;
-    if (blockIdx.x == 0 && threadIdx.x == 0) ctl->work[0] = 0;
+    if (blockIdx.x == 0 && threadIdx.x == 0) ctl->work[0].v = 0;
     if (P.lc && blockIdx.x == 0) {
         // Label-correcting: the next relaxation appends the frontier after it
         // into slot cur, whose frontier this round's relaxation has consumed.
@@ -1345,6 +1358,7 @@ __device__ void cupdate_phase(const RoundParams& P, unsigned char* s_dyn, u32 r)
     Acc an = {kInf64, kInf64, 0, 0, 0};
     WarpQueue qf = {s_qf + wib * kQCap, 0}, qa = {s_qa + wib * kQCap, 0};
     // First item per warp is static (no atomic); the rest are pulled.
+    u32 left = 0;
     for (u32 item = static_item(wib); item < total;) {
         if (item < w.tiles)
             cup_small<MULTI, L, TAIL>(P, s_st[wib], item, w.ts, nas, r, cur, lane,
@@ -1356,17 +1370,15 @@ __device__ void cupdate_phase(const RoundParams& P, unsigned char* s_dyn, u32 r)
             snap_frontier<L>(P, item - w.tiles - w.parts, nxt, sfs, sfh, lane);
         __syncwarp();
         if (total <= nwarps) break;                // the static items were all
-        u32 next = 0;
-        if (lane == 0) next = atomicAdd(&ctl->work[1], 1u) + nwarps;
-        item = __shfl_sync(kFull, next, 0);
+        item = next_item(&ctl->work[1].v, item, left, total, nwarps, lane);
     }
     // (Label-correcting: qf carries the vertices fixed this round, to FX.)
-    if (P.lc) wq_flush2(P, qf, &ctl->nFX[nxt], P.L.FX[nxt], qa, &ctl->nAS[nxt], P.L.AS[nxt], lane);
-    else wq_flush2(P, qf, &ctl->nFS[nxt], P.L.FS[nxt], qa, &ctl->nAS[nxt], P.L.AS[nxt], lane);
     a.fmin_d = an.fmin_d;
     a.fmin_t = an.fmin_t;
     a.nfix = an.nfix;
-    flush<MULTI, L::kNarrow>(P, nxt, nxt, a, lane, 1, 2);
+    end_phase<MULTI, L::kNarrow>(P, nxt, nxt, a, 1, 2, qf, P.lc ? &ctl->nFX[nxt] : &ctl->nFS[nxt],
+                                 P.lc ? P.L.FX[nxt] : P.L.FS[nxt], qa, &ctl->nAS[nxt],
+                                 P.L.AS[nxt], lane, wib);
 }
 
 template <bool MULTI, class L>
@@ -1633,7 +1645,7 @@ __global__ void k_start(RoundParams P, u32 first, u32 count, u32 max_rounds, u32
     }
     __syncthreads();
     if (threadIdx.x == 0) {
-        ctl->stats[4] += count;       // the sources are fixed
+        ctl->stats[4].v += count;       // the sources are fixed
         if (s_run) {
             ctl->status = kRunning;
             ctl->running += s_run;

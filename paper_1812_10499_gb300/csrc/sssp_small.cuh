@@ -856,17 +856,17 @@ __global__ void __launch_bounds__(kSmallThreads, 1)
         const u64 o = warp_sum64(a.out), i = warp_sum64(a.in), ac = warp_sum64(a.act),
                   fr = warp_sum64(a.front);
         if (lane == 0) {
-            if (o) atomicAdd(&ctl->stats[0], o);
-            if (i) atomicAdd(&ctl->stats[1], i);
-            if (ac) atomicAdd(&ctl->stats[2], ac);
-            if (fr) atomicAdd(&ctl->stats[3], fr);
+            if (o) atomicAdd(&ctl->stats[0].v, o);
+            if (i) atomicAdd(&ctl->stats[1].v, i);
+            if (ac) atomicAdd(&ctl->stats[2].v, ac);
+            if (fr) atomicAdd(&ctl->stats[3].v, fr);
         }
     }
     if (lead) {
-        ctl->stats[4] += reached;
+        ctl->stats[4].v += reached;
         ctl->round = r;
         ctl->cup_only = cup_only ? 1u : 0u;
-        ctl->work[0] = 0;
+        ctl->work[0].v = 0;
         u32 st = kRunning;
         if (end_status != kRunning) {
             iv->rounds = r - start_round;
@@ -882,7 +882,7 @@ __global__ void __launch_bounds__(kSmallThreads, 1)
             iv->minD[cu] = minD == S::kInf ? kInf64 : (u64)minD;
             iv->thr[cu] = thr == S::kInf ? kInf64 : (u64)thr;
             iv->nfix[cu ^ 1u] = 0;
-            ctl->work[1] = 0;
+            ctl->work[1].v = 0;
             ctl->done_ctas = 0;
         }
         if (P.cond) cudaGraphSetConditional(P.cond, (st == kRunning && r <= stop_round) ? 1u : 0u);
