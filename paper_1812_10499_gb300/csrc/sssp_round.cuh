@@ -253,10 +253,12 @@ __device__ __forceinline__ u32 warp_incl_scan(u32 x, u32 lane) {
     return x;
 }
 
+// Warp minimum, to every lane: the upper halves, then the lower halves of the
+// lanes that hold the least upper half.
 __device__ __forceinline__ u64 warp_min64(u64 v) {
-#pragma unroll
-    for (u32 d = 16; d >= 1; d >>= 1) v = umin64(v, __shfl_xor_sync(kFull, v, d));
-    return v;
+    const u32 hi = __reduce_min_sync(kFull, (u32)(v >> 32));
+    const u32 lo = __reduce_min_sync(kFull, (u32)(v >> 32) == hi ? (u32)v : kFull);
+    return ((u64)hi << 32) | lo;
 }
 __device__ __forceinline__ u64 warp_sum64(u64 v) {
 #pragma unroll
@@ -389,31 +391,80 @@ struct Acc {
     u64 edges, visits;
     u32 nfix;               // vertices fixed (single-query mode)
 };
+__device__ __forceinline__ Acc make_acc() { return Acc{kInf64, kInf64, 0, 0, 0}; }
 
 __device__ __forceinline__ void atomic_min_checked(u64* p, u64 v) {
     if (v < ld_volatile(p)) atomicMin(p, v);
 }
 
-// Fold one unfixed vertex's (D, D + outWeight) into the minima of `slot`.
-template <bool MULTI>
-__device__ __forceinline__ void fold(const RoundParams& P, u32 inst, u32 slot, u64 d, u64 t,
-                                     Acc& a) {
-    if (MULTI) {
+// Several queries: the CTA's folds and fixed counts by query, in shared memory.
+// A warp's vertices belong to many queries, and all warps of the grid fold into
+// the same few scalars: folded there one by one (a load and perhaps an atomic
+// each), 4 sources on R-MAT 18 took 2.5 times as long in the relaxation as one
+// query with the same work.  Slots beyond the cache fold in global memory.
+constexpr u32 kInstCache = 1024;
+template <class D>
+struct InstCache {
+    D mind[kInstCache], mint[kInstCache];
+    u32 nfix[kInstCache];
+};
+template <bool MULTI, class L>
+__device__ __forceinline__ InstCache<typename L::Term>* inst_cache(const RoundParams& P) {
+    if constexpr (MULTI) {
+        __shared__ InstCache<typename L::Term> c;
+        const u32 n = min(P.ctl->ninst, kInstCache);
+        for (u32 i = threadIdx.x; i < n; i += blockDim.x) {
+            c.mind[i] = c.mint[i] = ~(typename L::Term)0;
+            c.nfix[i] = 0;
+        }
+        __syncthreads();
+        return &c;
+    }
+    return nullptr;
+}
+template <class D>
+__device__ __forceinline__ void inst_fold(const RoundParams& P, InstCache<D>* ic, u32 inst,
+                                          u32 slot, u64 d, u64 t) {
+    if (inst < kInstCache) {
+        if ((D)d < ic->mind[inst]) atomicMin(&ic->mind[inst], (D)d);
+        if ((D)t < ic->mint[inst]) atomicMin(&ic->mint[inst], (D)t);
+    } else {
         atomic_min_checked(&P.ivar[inst].minD[slot], d);
         atomic_min_checked(&P.ivar[inst].thr[slot], t);
-    } else {
-        a.fmin_d = umin64(a.fmin_d, d);
-        a.fmin_t = umin64(a.fmin_t, t);
     }
+}
+template <class D>
+__device__ __forceinline__ void inst_count(const RoundParams& P, InstCache<D>* ic, u32 inst,
+                                           u32 nfix_slot) {
+    if (inst < kInstCache) atomicAdd(&ic->nfix[inst], 1u);
+    else atomicAdd(&P.ivar[inst].nfix[nfix_slot], 1u);
+}
+// End of the phase, after a __syncthreads.
+template <class D>
+__device__ __forceinline__ void inst_send(const RoundParams& P, const InstCache<D>* ic, u32 slot,
+                                          u32 nfix_slot) {
+    const u32 n = min(P.ctl->ninst, kInstCache);
+    for (u32 i = threadIdx.x; i < n; i += blockDim.x) {
+        InstVar* v = P.ivar + i;
+        if (ic->mind[i] != ~(D)0) atomic_min_checked(&v->minD[slot], ic->mind[i]);
+        if (ic->mint[i] != ~(D)0) atomic_min_checked(&v->thr[slot], ic->mint[i]);
+        if (ic->nfix[i]) atomicAdd(&v->nfix[nfix_slot], ic->nfix[i]);
+    }
+}
+
+// Fold one unfixed vertex's (D, D + outWeight) into the minima.
+__device__ __forceinline__ void fold(u64 d, u64 t, Acc& a) {
+    a.fmin_d = umin64(a.fmin_d, d);
+    a.fmin_t = umin64(a.fmin_t, t);
 }
 
 // End of a phase: the warps' remaining list entries, folds and counters leave
 // together, with one atomic per word and CTA (all threads of the CTA).  The
 // words are shared by the whole grid, and an atomic on one word takes about 4
 // cycles of its L2 slice: one per warp, from 3648 warps, would take 7 us a word.
-template <bool MULTI, bool NARROW>
-__device__ __forceinline__ void end_phase(const RoundParams& P, u32 slot, u32 nfix_slot,
-                                          const Acc& a, u32 stat_edges, u32 stat_visits,
+template <bool MULTI, bool NARROW, class D>
+__device__ __forceinline__ void end_phase(const RoundParams& P, InstCache<D>* ic, u32 slot,
+                                          u32 nfix_slot, const Acc& a, u32 stat_edges, u32 stat_visits,
                                           const WarpQueue& q0, u32* c0, u32* l0,
                                           const WarpQueue& q1, u32* c1, u32* l1, u32 lane,
                                           u32 wib) {
@@ -447,6 +498,7 @@ __device__ __forceinline__ void end_phase(const RoundParams& P, u32 slot, u32 nf
         s_nfix[wib] = nf;
     }
     __syncthreads();
+    if (MULTI) inst_send(P, ic, slot, nfix_slot);
     const bool in = lane < kWarps;
     if (wib == 0) {
         const u32 n0 = __reduce_add_sync(kFull, in ? s_cnt[0][lane] : 0u);
@@ -739,8 +791,9 @@ __device__ __forceinline__ void relax_issue(const RoundParams& P,
 // are exact without knowing which candidate won.  A target whose D was
 // infinite is newly discovered and joins the active set.
 template <bool MULTI, class L>
-__device__ __forceinline__ void relax_consume(const RoundParams& P, u32 cur, Acc& a, WarpQueue& q,
-                                              WarpQueue& qf, Pend& pd, u32 lane) {
+__device__ __forceinline__ void relax_consume(const RoundParams& P, InstCache<typename L::Term>* ic,
+                                              u32 cur, Acc& a, WarpQueue& q, WarpQueue& qf,
+                                              Pend& pd, u32 lane) {
     if (!pd.any) return;
     pd.any = false;
     const u32 nxt = cur ^ 1u;
@@ -762,7 +815,9 @@ __device__ __forceinline__ void relax_consume(const RoundParams& P, u32 cur, Acc
                 none = ow == kNoOutW;
             }
             const u64 dd = pd.cand[i] >> (L::kNarrow ? 32u : P.vbits);
-            fold<MULTI>(P, pd.inst[i], cur, dd, none ? P.dinf : dd + ow, a);
+            const u64 t = none ? P.dinf : dd + ow;
+            if (MULTI) inst_fold(P, ic, pd.inst[i], cur, dd, t);
+            else fold(dd, t, a);
         }
         const bool sm = fresh && !hub;
         wq_push(P, q, &P.ctl->nAS[cur], P.L.AS[cur], sm, pd.gy[i], lane);
@@ -784,7 +839,7 @@ __device__ __forceinline__ void relax_consume(const RoundParams& P, u32 cur, Acc
             if (chg) {
                 const InstDesc& d = MULTI ? P.idesc[pd.inst[i]] : P.g;
                 odeg = d.out_off[pd.yl[i] + 1] - d.out_off[pd.yl[i]];
-                if (MULTI) atomicAdd(&P.ivar[pd.inst[i]].nfix[nxt], 1u);
+                if (MULTI) inst_count(P, ic, pd.inst[i], nxt);
                 else a.nfix++;
             }
             const bool fs = chg && odeg <= P.hub;
@@ -795,7 +850,7 @@ __device__ __forceinline__ void relax_consume(const RoundParams& P, u32 cur, Acc
 }
 
 template <bool MULTI, class L>
-__device__ void relax_small(const RoundParams& P, WarpStage<typename L::RSlot>& st, u32 t,
+__device__ void relax_small(const RoundParams& P, InstCache<typename L::Term>* ic, WarpStage<typename L::RSlot>& st, u32 t,
                             u32 ts, u32 nfs, u32 cur, u32 lane, Acc& a, WarpQueue& q,
                             WarpQueue& qf, Pend& pd) {
     const u32 idx = (t << ts) + lane;
@@ -827,14 +882,14 @@ __device__ void relax_small(const RoundParams& P, WarpStage<typename L::RSlot>& 
                                      lane);
         },
         [&](u32 bb, u32 as, u32 ds) {
-            relax_consume<MULTI, L>(P, cur, a, q, qf, pd, lane);
+            relax_consume<MULTI, L>(P, ic, cur, a, q, qf, pd, lane);
             relax_issue<MULTI, L>(P, st, as, ds, min(kB, tl.total - bb * kB), cur, true, dx, xloc,
                                   gbase, inst, a, pd, lane);
         });
 }
 
 template <bool MULTI, class L>
-__device__ void relax_hub(const RoundParams& P, WarpStage<typename L::RSlot>& st, u32 item, u32 ps,
+__device__ void relax_hub(const RoundParams& P, InstCache<typename L::Term>* ic, WarpStage<typename L::RSlot>& st, u32 item, u32 ps,
                           u32 nfh, u32 cur, u32 lane, Acc& a, WarpQueue& q, WarpQueue& qf,
                           Pend& pd) {
     const uint2* FH = P.L.FH[cur];
@@ -861,7 +916,7 @@ __device__ void relax_hub(const RoundParams& P, WarpStage<typename L::RSlot>& st
             issue_dc<MULTI, L, true>(P, st, as, ds, min(kB, n - bb * kB), cur, d.base, false, lane);
         },
         [&](u32 bb, u32 as, u32 ds) {
-            relax_consume<MULTI, L>(P, cur, a, q, qf, pd, lane);
+            relax_consume<MULTI, L>(P, ic, cur, a, q, qf, pd, lane);
             relax_issue<MULTI, L>(P, st, as, ds, min(kB, n - bb * kB), cur, false, dx, xloc,
                                   d.base, inst, a, pd, lane);
         });
@@ -884,6 +939,7 @@ __device__ void relax_phase(const RoundParams& P, unsigned char* s_dyn, u32 r) {
     Stage* s_st = reinterpret_cast<Stage*>(s_dyn);
     u32* s_q = reinterpret_cast<u32*>(s_dyn + sizeof(Stage) * kWarps);
     Ctl* ctl = P.ctl;
+    auto* const ic = inst_cache<MULTI, L>(P);
     const u32 cur = r & 1u, nxt = cur ^ 1u;
     const u32 lane = threadIdx.x & 31u, wib = threadIdx.x >> 5;
 
@@ -924,7 +980,7 @@ __device__ void relax_phase(const RoundParams& P, unsigned char* s_dyn, u32 r) {
     const u32 nfx = (P.lc || P.win) ? min(ctl->nFX[cur], P.L.capS) : 0u;
     const u32 total = w.tiles + w.parts + ((nfx + 31) >> 5);
 
-    Acc a = {kInf64, kInf64, 0, 0, 0};
+    Acc a = make_acc();
     WarpQueue q = {s_q + wib * kQCap, 0};
     WarpQueue qf = {s_q + (kWarps + wib) * kQCap, 0};   // label-correcting next frontier
     Pend pd;
@@ -934,9 +990,9 @@ __device__ void relax_phase(const RoundParams& P, unsigned char* s_dyn, u32 r) {
     u32 left = 0;
     for (u32 item = static_item(wib); item < total;) {
         if (item < w.tiles) {
-            relax_small<MULTI, L>(P, s_st[wib], item, w.ts, nfs, cur, lane, a, q, qf, pd);
+            relax_small<MULTI, L>(P, ic, s_st[wib], item, w.ts, nfs, cur, lane, a, q, qf, pd);
         } else if (item < w.tiles + w.parts) {
-            relax_hub<MULTI, L>(P, s_st[wib], item - w.tiles, w.ps, nfh, cur, lane, a, q, qf, pd);
+            relax_hub<MULTI, L>(P, ic, s_st[wib], item - w.tiles, w.ps, nfh, cur, lane, a, q, qf, pd);
         } else {
             const u32 idx = (item - w.tiles - w.parts) * 32 + lane;
             if (idx < nfx) {
@@ -947,8 +1003,8 @@ __device__ void relax_phase(const RoundParams& P, unsigned char* s_dyn, u32 r) {
         if (total <= nwarps) break;                // the static items were all
         item = next_item(&ctl->work[0].v, item, left, total, nwarps, lane);
     }
-    relax_consume<MULTI, L>(P, cur, a, q, qf, pd, lane);
-    end_phase<MULTI, L::kNarrow>(P, cur, nxt, a, 0, 3, q, &ctl->nAS[cur], P.L.AS[cur], qf,
+    relax_consume<MULTI, L>(P, ic, cur, a, q, qf, pd, lane);
+    end_phase<MULTI, L::kNarrow>(P, ic, cur, nxt, a, 0, 3, q, &ctl->nAS[cur], P.L.AS[cur], qf,
                                  &ctl->nFS[nxt], P.L.FS[nxt], lane, wib);
 }
 
@@ -1010,7 +1066,7 @@ __device__ __forceinline__ u64 decide(const RoundParams& P, u64 dy, u64 cy, u64 
 // faster, and with the wide layout's 64-bit terms the atomics cost 1.4% on
 // the 4096^2 grid, so both keep the scan.
 template <bool MULTI, class L, bool SHATOM = false>
-__device__ void cup_small(const RoundParams& P, WarpStage<typename L::CSlot>& st, u32 t, u32 ts,
+__device__ void cup_small(const RoundParams& P, InstCache<typename L::Term>* ic, WarpStage<typename L::CSlot>& st, u32 t, u32 ts,
                           u32 nas, u32 r, u32 cur, u32 lane, u64* smin, u64 thr0, u64 minD0,
                           Acc& a, Acc& an, WarpQueue& qf, WarpQueue& qa) {
     const u32 nxt = cur ^ 1u;
@@ -1027,8 +1083,8 @@ __device__ void cup_small(const RoundParams& P, WarpStage<typename L::CSlot>& st
         gbase = d.base;
         in_adj = d.in_adj;
         if (MULTI) {
-            thr = ld_volatile(&P.ivar[inst].thr[cur]);
-            minD = ld_volatile(&P.ivar[inst].minD[cur]);
+            thr = P.ivar[inst].thr[cur];          // (stable during this phase)
+            minD = P.ivar[inst].minD[cur];
         }
         yloc = g - (u32)gbase;
         ib = d.in_off[yloc];
@@ -1128,16 +1184,18 @@ __device__ void cup_small(const RoundParams& P, WarpStage<typename L::CSlot>& st
     else wq_push(P, qf, &P.ctl->nFS[nxt], P.L.FS[nxt], fs, g, lane);
     if (fx && !fs) put_hub(P, &P.ctl->FHpk[nxt], P.L.FH[nxt], P.L.FC[nxt], g, odeg);
     wq_push(P, qa, &P.ctl->nAS[nxt], P.L.AS[nxt], sv, g, lane);
+    const u64 tsum = outw == kNoOutW ? P.dinf : dy + outw;
     if (MULTI) {
-        if (fx) atomicAdd(&P.ivar[inst].nfix[nxt], 1u);
+        if (fx) inst_count(P, ic, inst, nxt);
+        if (sv) inst_fold(P, ic, inst, nxt, dy, tsum);
     } else {
         an.nfix += fx;
+        if (sv) fold(dy, tsum, an);
     }
-    if (sv) fold<MULTI>(P, inst, nxt, dy, outw == kNoOutW ? P.dinf : dy + outw, an);
 }
 
 template <bool MULTI, class L>
-__device__ void cup_hub(const RoundParams& P, WarpStage<typename L::CSlot>& st, u32 item, u32 ps,
+__device__ void cup_hub(const RoundParams& P, InstCache<typename L::Term>* ic, WarpStage<typename L::CSlot>& st, u32 item, u32 ps,
                         u32 nah, u32 r, u32 cur, u32 lane, u64 thr0, u64 minD0, Acc& a, Acc& an) {
     const u32 nxt = cur ^ 1u;
     const u32 c = item >> ps, part = item & ((1u << ps) - 1u);
@@ -1149,8 +1207,8 @@ __device__ void cup_hub(const RoundParams& P, WarpStage<typename L::CSlot>& st, 
     const InstDesc& d = desc_of<MULTI>(P, g, inst);
     u64 thr = thr0, minD = minD0;
     if (MULTI) {
-        thr = ld_volatile(&P.ivar[inst].thr[cur]);
-        minD = ld_volatile(&P.ivar[inst].minD[cur]);
+        thr = P.ivar[inst].thr[cur];
+        minD = P.ivar[inst].minD[cur];
     }
     const u32 yloc = g - (u32)d.base;
     const u64 ib = d.in_off[yloc], ie = d.in_off[yloc + 1];
@@ -1215,7 +1273,9 @@ __device__ void cup_hub(const RoundParams& P, WarpStage<typename L::CSlot>& st, 
         if (P.lc || P.win) put_small(P, P.L.FX[nxt], atomicAdd(&P.ctl->nFX[nxt], 1u), g);
     } else {
         put_hub(P, &P.ctl->AHpk[nxt], P.L.AH[nxt], P.L.AC[nxt], g, ie - ib);
-        fold<MULTI>(P, inst, nxt, dy, outw == kNoOutW ? P.dinf : dy + outw, an);
+        const u64 t = outw == kNoOutW ? P.dinf : dy + outw;
+        if (MULTI) inst_fold(P, ic, inst, nxt, dy, t);
+        else fold(dy, t, an);
     }
     if (P.win) {
         front = P.chg[g] != 0 && (fix || dy < win_limit(minD, P.delta));
@@ -1228,7 +1288,7 @@ __device__ void cup_hub(const RoundParams& P, WarpStage<typename L::CSlot>& st, 
         const u64 odeg = d.out_off[yloc + 1] - d.out_off[yloc];
         if (odeg <= P.hub) put_small(P, P.L.FS[nxt], atomicAdd(&P.ctl->nFS[nxt], 1u), g);
         else put_hub(P, &P.ctl->FHpk[nxt], P.L.FH[nxt], P.L.FC[nxt], g, odeg);
-        if (MULTI) atomicAdd(&P.ivar[inst].nfix[nxt], 1u);
+        if (MULTI) inst_count(P, ic, inst, nxt);
         else an.nfix++;
     }
 }
@@ -1321,6 +1381,7 @@ __device__ void cupdate_phase(const RoundParams& P, unsigned char* s_dyn, u32 r)
     u32* s_qf = reinterpret_cast<u32*>(s_min + kWarps * 32);
     u32* s_qa = s_qf + kWarps * kQCap;
     Ctl* ctl = P.ctl;
+    auto* const ic = inst_cache<MULTI, L>(P);
     const u32 cur = r & 1u, nxt = cur ^ 1u;
     const u32 lane = threadIdx.x & 31u, wib = threadIdx.x >> 5;
     if (blockIdx.x == 0 && threadIdx.x == 0) ctl->work[0].v = 0;
@@ -1354,17 +1415,16 @@ __device__ void cupdate_phase(const RoundParams& P, unsigned char* s_dyn, u32 r)
         minD = P.ivar[0].minD[cur];
     }
 
-    Acc a = {kInf64, kInf64, 0, 0, 0};
-    Acc an = {kInf64, kInf64, 0, 0, 0};
+    Acc a = make_acc(), an = make_acc();
     WarpQueue qf = {s_qf + wib * kQCap, 0}, qa = {s_qa + wib * kQCap, 0};
     // First item per warp is static (no atomic); the rest are pulled.
     u32 left = 0;
     for (u32 item = static_item(wib); item < total;) {
         if (item < w.tiles)
-            cup_small<MULTI, L, TAIL>(P, s_st[wib], item, w.ts, nas, r, cur, lane,
+            cup_small<MULTI, L, TAIL>(P, ic, s_st[wib], item, w.ts, nas, r, cur, lane,
                                       s_min + wib * 32, thr, minD, a, an, qf, qa);
         else if (item < w.tiles + w.parts)
-            cup_hub<MULTI, L>(P, s_st[wib], item - w.tiles, w.ps, nah, r, cur, lane, thr, minD, a,
+            cup_hub<MULTI, L>(P, ic, s_st[wib], item - w.tiles, w.ps, nah, r, cur, lane, thr, minD, a,
                               an);
         else
             snap_frontier<L>(P, item - w.tiles - w.parts, nxt, sfs, sfh, lane);
@@ -1376,7 +1436,7 @@ __device__ void cupdate_phase(const RoundParams& P, unsigned char* s_dyn, u32 r)
     a.fmin_d = an.fmin_d;
     a.fmin_t = an.fmin_t;
     a.nfix = an.nfix;
-    end_phase<MULTI, L::kNarrow>(P, nxt, nxt, a, 1, 2, qf, P.lc ? &ctl->nFX[nxt] : &ctl->nFS[nxt],
+    end_phase<MULTI, L::kNarrow>(P, ic, nxt, nxt, a, 1, 2, qf, P.lc ? &ctl->nFX[nxt] : &ctl->nFS[nxt],
                                  P.lc ? P.L.FX[nxt] : P.L.FS[nxt], qa, &ctl->nAS[nxt],
                                  P.L.AS[nxt], lane, wib);
 }
