@@ -530,17 +530,27 @@ int init_single_context(sssp_graph* h) {
     return SSSP_OK;
 }
 
+// Checks a CSR and finds its largest weight.  The edges are read once, in loops
+// over the plain arrays that the compiler can vectorise (largest target, least and
+// largest weight); only a graph that fails is walked edge by edge, for the
+// first fault.
 int validate_csr(u32 n, u64 m, const u64* off, const u32* idx, const u32* w, u32* wmax) {
     if (!off || (m && (!idx || !w))) return SSSP_E_INVAL;
     if (off[0] != 0 || off[n] != m) return SSSP_E_INVAL;
-    u32 mx = 0;
-    for (u32 u = 0; u < n; ++u)
-        if (off[u + 1] < off[u]) return SSSP_E_INVAL;
+    u32 falls = 0;
+    for (u32 u = 0; u < n; ++u) falls |= off[u + 1] < off[u];
+    if (falls) return SSSP_E_INVAL;
+    u32 top = 0, least = 0xFFFFFFFFu, mx = 0;
+    for (u64 k = 0; k < m; ++k) top = idx[k] > top ? idx[k] : top;
     for (u64 k = 0; k < m; ++k) {
-        if (idx[k] >= n) return SSSP_E_INVAL;
-        if (w[k] == 0) return SSSP_E_ZERO_WEIGHT;
-        mx = std::max(mx, w[k]);
+        least = w[k] < least ? w[k] : least;
+        mx = w[k] > mx ? w[k] : mx;
     }
+    if (m && (top >= n || least == 0))
+        for (u64 k = 0; k < m; ++k) {
+            if (idx[k] >= n) return SSSP_E_INVAL;
+            if (w[k] == 0) return SSSP_E_ZERO_WEIGHT;
+        }
     *wmax = mx;
     return SSSP_OK;
 }
@@ -566,11 +576,26 @@ void strip_loops(u32 n, const u64* off, const u32* idx, const u32* w, std::vecto
     o2[n] = i2.size();
 }
 
-bool has_loop(u32 n, const u64* off, const u32* idx) {
-    for (u32 u = 0; u < n; ++u)
-        for (u64 k = off[u]; k < off[u + 1]; ++k)
-            if (idx[k] == u) return true;
-    return false;
+// Whether the uploaded out-edges hold a self-loop (waits for the stream).
+int has_loop(sssp_graph* h, u32 n, bool* found) {
+    Pool tmp;
+    tmp.al = h->gpool.al;
+    u32* flag = nullptr;
+    u32 v = 0;
+    RC(tmp.get(&flag, 1));
+    cudaError_t e = cudaMemsetAsync(flag, 0, sizeof(u32), h->stream);
+    if (e == cudaSuccess) {
+        k_find_loop<<<h->grid, kThreads, 0, h->stream>>>(h->out_off, h->out_adj, n, flag);
+        e = cudaGetLastError();
+    }
+    if (e == cudaSuccess)
+        e = cudaMemcpyAsync(&v, flag, sizeof(u32), cudaMemcpyDeviceToHost, h->stream);
+    const cudaError_t es = cudaStreamSynchronize(h->stream);
+    tmp.release();
+    CK(e);
+    CK(es);
+    *found = v != 0;
+    return SSSP_OK;
 }
 
 int upload_adj(sssp_graph* h, const u32* idx, const u32* w, u64 m, uint2* adj) {
@@ -598,27 +623,17 @@ int upload_adj(sssp_graph* h, const u32* idx, const u32* w, u64 m, uint2* adj) {
     return rc;
 }
 
+// Builds the graph on the device from arrays that sssp_create has checked
+// (wmax: their largest weight).
 int create_impl(sssp_graph* h, u32 n, u64 m, const u64* row_ptr, const u32* col, const u32* w,
-                const u64* col_ptr, const u32* row, const u32* w_in) {
-    u32 wmax = 0;
-    RC(validate_csr(n, m, row_ptr, col, w, &wmax));
+                const u64* col_ptr, const u32* row, const u32* w_in, u32 wmax) {
     const bool csc_given = col_ptr || row || w_in;
-    if (csc_given) {
-        if (!(col_ptr && (m == 0 || (row && w_in)))) return SSSP_E_INVAL;
-        u32 wmax2 = 0;
-        RC(validate_csr(n, m, col_ptr, row, w_in, &wmax2));
-        if (wmax2 != wmax) return SSSP_E_INVAL;
-    }
     h->vbits = std::max<u32>(1, bits_for((u64)n - 1));
     h->dinf = (~0ull) >> h->vbits;
-    // Every finite quantity of a round (D, C, lb + w, D + outWeight) stays
-    // below n * wmax; it must stay below the infinity of the packed word.
-    if (wmax && (unsigned __int128)n * wmax >= (unsigned __int128)h->dinf) return SSSP_E_OVERFLOW;
     h->wmax = wmax;
     // Compact records hold 31-bit lower bounds: every finite distance
     // (at most (n - 1) * wmax) must stay below 2^31 - 1.
     const bool fits = (unsigned __int128)n * wmax < kNarrowLimit;
-    if (h->opt.layout == SSSP_LAYOUT_COMPACT && !fits) return SSSP_E_OVERFLOW;
     h->narrow = fits && h->opt.layout != SSSP_LAYOUT_WIDE;
     if (h->narrow) {
         // The compact kernels keep the distance in the upper half of the
@@ -626,25 +641,6 @@ int create_impl(sssp_graph* h, u32 n, u64 m, const u64* row_ptr, const u32* col,
         h->vbits = 32;
         h->dinf = (~0ull) >> 32;
     }
-
-    std::vector<u64> o2, c2;
-    std::vector<u32> i2, w2, r2, wi2;
-    if (has_loop(n, row_ptr, col)) {
-        strip_loops(n, row_ptr, col, w, o2, i2, w2);
-        row_ptr = o2.data();
-        col = i2.data();
-        w = w2.data();
-        m = o2[n];
-        if (csc_given) {
-            strip_loops(n, col_ptr, row, w_in, c2, r2, wi2);
-            col_ptr = c2.data();
-            row = r2.data();
-            w_in = wi2.data();
-            if (c2[n] != m) return SSSP_E_INVAL;
-        }
-    }
-    h->n = n;
-    h->m = m;
 
     CK(cudaStreamCreateWithFlags(&h->stream, cudaStreamNonBlocking));
     h->grid = occupancy_grid(h->device, h->opt);
@@ -664,6 +660,27 @@ int create_impl(sssp_graph* h, u32 n, u64 m, const u64* row_ptr, const u32* col,
     CK(cudaMemcpyAsync(h->out_off, row_ptr, sizeof(u64) * ((size_t)n + 1), cudaMemcpyHostToDevice,
                        h->stream));
     RC(upload_adj(h, col, w, m, h->out_adj));
+    // Self-loops (rare) are dropped on the host and the edges uploaded again.
+    std::vector<u64> o2, c2;
+    std::vector<u32> i2, w2, r2, wi2;
+    bool loops = false;
+    RC(has_loop(h, n, &loops));
+    if (loops) {
+        strip_loops(n, row_ptr, col, w, o2, i2, w2);
+        m = o2[n];
+        if (csc_given) {
+            strip_loops(n, col_ptr, row, w_in, c2, r2, wi2);
+            col_ptr = c2.data();
+            row = r2.data();
+            w_in = wi2.data();
+            if (c2[n] != m) return SSSP_E_INVAL;
+        }
+        CK(cudaMemcpyAsync(h->out_off, o2.data(), sizeof(u64) * ((size_t)n + 1),
+                           cudaMemcpyHostToDevice, h->stream));
+        RC(upload_adj(h, i2.data(), w2.data(), m, h->out_adj));
+    }
+    h->n = n;
+    h->m = m;
     if (csc_given) {
         CK(cudaMemcpyAsync(h->in_off, col_ptr, sizeof(u64) * ((size_t)n + 1),
                            cudaMemcpyHostToDevice, h->stream));
@@ -1065,9 +1082,13 @@ int sssp_create(uint32_t n, uint64_t m, const uint64_t* row_ptr, const uint32_t*
         o.hub_degree > (1u << 20) || o.chunk_edges > (1u << 20) ||
         o.block_threads != kThreads || (o.alloc == nullptr) != (o.free == nullptr))
         return SSSP_E_INVAL;
+    u32 wmax = 0;
     {
         // Host-side checks first: no device is touched for a malformed graph.
-        u32 wmax = 0, wmax2 = 0;
+        // (Every finite quantity of a round -- D, C, lb + w, D + outWeight --
+        // stays below n * wmax; it must stay below the infinity of the packed
+        // word.)
+        u32 wmax2 = 0;
         RC(validate_csr(n, m, reinterpret_cast<const u64*>(row_ptr), col, w, &wmax));
         if (col_ptr || row || w_in) {
             if (!(col_ptr && (m == 0 || (row && w_in)))) return SSSP_E_INVAL;
@@ -1096,7 +1117,7 @@ int sssp_create(uint32_t n, uint64_t m, const uint64_t* row_ptr, const uint32_t*
     {
         DeviceGuard dg(dev);
         rc = create_impl(h, n, m, reinterpret_cast<const u64*>(row_ptr), col, w,
-                         reinterpret_cast<const u64*>(col_ptr), row, w_in);
+                         reinterpret_cast<const u64*>(col_ptr), row, w_in, wmax);
         if (rc != SSSP_OK) destroy_impl(h);
     }
     if (rc != SSSP_OK) {

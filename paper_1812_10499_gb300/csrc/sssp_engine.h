@@ -51,6 +51,7 @@ __global__ void k_finalize(const VRec* rec, const VRecN* recn, const int* frec, 
                            u64* lower);
 __global__ void k_finalize_multi(RoundParams P, u64 nrec, u64* dist);
 __global__ void k_interleave(const u32* col, const u32* w, u64 m, uint2* adj);
+__global__ void k_find_loop(const u64* out_off, const uint2* out_adj, u32 n, u32* flag);
 __global__ void k_count_in(const uint2* adj, u64 m, u64* cnt);
 __global__ void k_scatter_in(const u64* out_off, const uint2* out_adj, u32 n, u64* cursor,
                              uint2* in_adj);

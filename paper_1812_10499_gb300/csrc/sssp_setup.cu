@@ -138,6 +138,18 @@ __global__ void k_interleave(const u32* col, const u32* w, u64 m, uint2* adj) {
         adj[i] = make_uint2(col[i], w[i]);
 }
 
+// Sets *flag when some out-edge leads back to its vertex (one warp per vertex).
+__global__ void k_find_loop(const u64* out_off, const uint2* out_adj, u32 n, u32* flag) {
+    const u32 lane = threadIdx.x & 31u;
+    for (u64 u = (blockIdx.x * (u64)blockDim.x + threadIdx.x) >> 5; u < n;
+         u += ((u64)gridDim.x * blockDim.x) >> 5) {
+        bool loop = false;
+        for (u64 k = out_off[u] + lane; k < out_off[u + 1]; k += 32)
+            loop = loop || out_adj[k].x == (u32)u;
+        if (__any_sync(kFull, loop) && lane == 0) *flag = 1u;
+    }
+}
+
 __global__ void k_count_in(const uint2* adj, u64 m, u64* cnt) {
     for (u64 i = blockIdx.x * (u64)blockDim.x + threadIdx.x; i < m;
          i += (u64)gridDim.x * blockDim.x)

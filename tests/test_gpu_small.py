@@ -80,3 +80,30 @@ def test_hand_over_between_the_kernels(sssp_lib, layout, tail_items, monkeypatch
     for g, s in ((gg.grid(60, 45, 1, 300, 3), 7), (gg.random_graph(3000, 5, 1, 60, 4), 1)):
         assert_parity(sssp_lib, g, s, layout=layout)
         assert_parity(sssp_lib, g, s, delta=20, layout=layout)
+
+
+@pytest.mark.parametrize("given_csc", [False, True])
+@pytest.mark.parametrize("where", ["first", "last", "every"])
+def test_self_loops_are_dropped(sssp_lib, given_csc, where):
+    """A loop at either end of the edge list, or at every vertex, with and
+    without the caller's CSC: the graph is the one without the loops."""
+    n = 333
+    base = gg.random_graph(n, 4, 1, 50, 8)
+    src, col, w = base.edges()
+    at = {"first": [0], "last": [n - 1], "every": list(range(n))}[where]
+    edges = list(zip(src.tolist(), col.tolist(), w.tolist()))
+    g = gg.from_edges(n, edges + [(v, v, 1) for v in at])
+    csc = {}
+    if given_csc:
+        s, c, ww = g.edges()
+        order = np.argsort(c, kind="stable")
+        ptr = np.concatenate([[0], np.cumsum(np.bincount(c, minlength=n))])
+        csc = dict(col_ptr=ptr.astype(np.uint64), row=s[order], w_in=ww[order])
+    h = sssp_lib.sssp_create(g.n, g.row_ptr, g.col, g.w, **csc)
+    try:
+        assert sssp_lib.sssp_num_edges(h) == base.m
+        out = sssp_lib.sssp_solve_ex(h, 5, parent=True)
+    finally:
+        sssp_lib.sssp_destroy(h)
+    ref = oracle.round_r(base, 5)
+    assert np.array_equal(out["dist"], ref.dist) and np.array_equal(out["parent"], ref.parent)
