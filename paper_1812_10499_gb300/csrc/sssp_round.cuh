@@ -658,16 +658,16 @@ __device__ __forceinline__ void issue_range_adj(WarpStage<S>& st, u32 s, const u
     }
 }
 
-// Starts gathering the neighbour states of the nb edges in adjacency slot
+// Starts gathering the target states of the nb out-edges in adjacency slot
 // as into state slot ds.  `base` is the record base of the edge's graph,
 // taken from the owning lane in multi-query mode.
-template <bool MULTI, class L, bool RELAX = false, class S>
+template <bool MULTI, class L, class S>
 __device__ __forceinline__ void issue_dc(const RoundParams& P, WarpStage<S>& st, u32 as, u32 ds,
                                          u32 nb, u32 cur, u64 base, bool per_owner, u32 lane) {
     typename L::Rec* rec = L::rec(P);
     // The relaxation of the compact label-setting round stages the 8-byte
     // filter word (relaxation bound, outWeight) instead of the record.
-    const bool filt = RELAX && L::kNarrow && P.gf != nullptr;
+    const bool filt = L::kNarrow && P.gf != nullptr;
 #pragma unroll
     for (u32 i = 0; i < kBI; ++i) {
         if (32 * i >= nb) break;                   // warp-uniform
@@ -679,6 +679,45 @@ __device__ __forceinline__ void issue_dc(const RoundParams& P, WarpStage<S>& st,
         const u32 gy = (u32)(ob + st.adj[as][idx].x);
         if (filt) cp_async_8(&st.dc[ds][idx], P.gf + gy);
         else st.dc[ds][idx].issue(rec + gy, cur);
+    }
+}
+
+// The largest in-edge weight that can matter to the Eq. (1) minimum of an
+// active vertex y, plus one (0: none can).  A fixed in-neighbour x has relaxed
+// its edge, so its term D[x] + w is D[y] or more; any other x has lb(x) >= minD.
+// So a term below D[y] needs minD + w < D[y], and the minimum never exceeds D[y]
+// (D[y] came over an in-edge from an x with lb(x) <= D[x]): the minimum over the
+// edges with w < D[y] - minD, and D[y], is the minimum over all.
+__device__ __forceinline__ u64 weight_limit(u64 dy, u64 minD) { return dy > minD ? dy - minD : 0; }
+
+// Starts gathering the source states of the nb in-edges in adjacency slot as
+// into state slot ds, of those edges whose weight is at most the owner's wtop;
+// the others get weight 0 (no edge has it) and are passed over.  The gathers are
+// what a large lower-bound phase waits on: 32 bytes of L2 per edge at random,
+// beside 8 bytes of adjacency in sequence.  On R-MAT 22 (weights to 255) 10-25%
+// of the in-edges are kept, 2.79 -> 2.65 ms a solve; on 128 random graphs (to
+// 1000) about half, 15.4 -> 14.0; 64 sources on R-MAT 18 16.9 -> 14.9.
+template <bool MULTI, class L, class S>
+__device__ __forceinline__ void issue_nbr(const RoundParams& P, WarpStage<S>& st, u32 as, u32 ds,
+                                          u32 nb, u32 cur, u64 base, u32 wtop, bool per_owner,
+                                          u32 lane) {
+    typename L::Rec* rec = L::rec(P);
+#pragma unroll
+    for (u32 i = 0; i < kBI; ++i) {
+        if (32 * i >= nb) break;                   // warp-uniform
+        const u32 idx = 32 * i + lane;
+        const bool ev = idx < nb;
+        u64 ob = base;
+        u32 top = wtop;
+        if (per_owner) {
+            const u32 own = ev ? st.own[as][idx] : 0u;
+            top = __shfl_sync(kFull, wtop, own);
+            if (MULTI) ob = __shfl_sync(kFull, base, own);
+        }
+        if (!ev) continue;
+        const uint2 e = st.adj[as][idx];
+        if (e.y <= top) st.dc[ds][idx].issue(rec + (u32)(ob + e.x), cur);
+        else st.adj[as][idx].y = 0u;
     }
 }
 
@@ -878,7 +917,7 @@ __device__ void relax_small(const RoundParams& P, InstCache<typename L::Term>* i
         (tl.total + kB - 1) / kB,
         [&](u32 bb, u32 s) { issue_tile_adj(st, tl, s, bb * kB, deg, lane); },
         [&](u32 bb, u32 as, u32 ds) {
-            issue_dc<MULTI, L, true>(P, st, as, ds, min(kB, tl.total - bb * kB), cur, gbase, true,
+            issue_dc<MULTI, L>(P, st, as, ds, min(kB, tl.total - bb * kB), cur, gbase, true,
                                      lane);
         },
         [&](u32 bb, u32 as, u32 ds) {
@@ -913,7 +952,7 @@ __device__ void relax_hub(const RoundParams& P, InstCache<typename L::Term>* ic,
         (n + kB - 1) / kB,
         [&](u32 bb, u32 s) { issue_range_adj(st, s, d.out_adj, cb + bb * kB, ce, lane); },
         [&](u32 bb, u32 as, u32 ds) {
-            issue_dc<MULTI, L, true>(P, st, as, ds, min(kB, n - bb * kB), cur, d.base, false, lane);
+            issue_dc<MULTI, L>(P, st, as, ds, min(kB, n - bb * kB), cur, d.base, false, lane);
         },
         [&](u32 bb, u32 as, u32 ds) {
             relax_consume<MULTI, L>(P, ic, cur, a, q, qf, pd, lane);
@@ -1100,19 +1139,24 @@ __device__ void cup_small(const RoundParams& P, InstCache<typename L::Term>* ic,
         if (L::kPred && !fix_now) fix_now = P.pcnt[g] == 0u;
         if (fix_now) deg = 0;                     // its in-edges are not read
     }
+    a.edges += deg;
+    const u64 lim = weight_limit(dy, minD);
+    const u32 wtop = (u32)umin64(lim - 1, kFull);
+    if (lim == 0) deg = 0;                        // none of its in-edges can matter
     // The owners' minima: 64-bit slots, or (compact layout, SHATOM) 32-bit
     // slots in their place.
     constexpr bool kAtom = SHATOM && L::kNarrow;
     u32* smin32 = reinterpret_cast<u32*>(smin);
-    if (kAtom) smin32[lane] = kInf31;
-    else smin[lane] = kInf64;
+    if (kAtom) smin32[lane] = (u32)dy;
+    else smin[lane] = dy;
     const typename L::Bounds bd = L::bounds(thr, minD);
     Tile tl = make_tile(st, deg, (u64)(in_adj + ib), lane);
     run_pipeline(
         (tl.total + kB - 1) / kB,
         [&](u32 b, u32 s) { issue_tile_adj(st, tl, s, b * kB, deg, lane); },
         [&](u32 b, u32 as, u32 ds) {
-            issue_dc<MULTI, L>(P, st, as, ds, min(kB, tl.total - b * kB), cur, gbase, true, lane);
+            issue_nbr<MULTI, L>(P, st, as, ds, min(kB, tl.total - b * kB), cur, gbase, wtop, true,
+                                lane);
         },
         [&](u32 b, u32 as, u32 ds) {
             const u32 nb = min(kB, tl.total - b * kB);
@@ -1128,11 +1172,13 @@ __device__ void cup_small(const RoundParams& P, InstCache<typename L::Term>* ic,
                     ob.minD = __shfl_sync(kFull, bd.minD, own);
                 }
                 typename L::Term val = L::kTermInf;
-                if (ev) val = L::term(P, st.dc[ds][sidx], cur, st.adj[as][sidx].y, ob);
+                const u32 w = ev ? st.adj[as][sidx].y : 0u;
+                if (w) val = L::term(P, st.dc[ds][sidx], cur, w, ob);
                 if (kAtom) {
-                    if (ev) atomicMin(smin32 + own, (u32)val);
+                    if (w) atomicMin(smin32 + own, (u32)val);
                     continue;
                 }
+                if (!__any_sync(kFull, w != 0)) continue;
                 // Min over the lanes sharing an owner (contiguous lanes; a
                 // segment starts at every owner change).
                 const u32 prev = __shfl_up_sync(kFull, own, 1);
@@ -1149,7 +1195,6 @@ __device__ void cup_small(const RoundParams& P, InstCache<typename L::Term>* ic,
                 __syncwarp();
             }
         });
-    a.edges += (lane == 0) ? tl.total : 0;
     __syncwarp();
 
     bool fix = false;
@@ -1220,28 +1265,31 @@ __device__ void cup_hub(const RoundParams& P, InstCache<typename L::Term>* ic, W
     // Cheaper rules first: every chunk of y takes the same decision (the
     // predecessor counts do not change during this phase).
     bool fix_now = false;
-    if (P.cheap)
-        fix_now = cheap_rules_fix(L::ld_dc(L::rec(P) + g, cur).x >> P.vbits, d.inw[yloc], thr,
-                                  minD);
+    const u64 dh = L::ld_dc(L::rec(P) + g, cur).x >> P.vbits;
+    if (P.cheap) fix_now = cheap_rules_fix(dh, d.inw[yloc], thr, minD);
     if (L::kPred && !fix_now) fix_now = P.pcnt[g] == 0u;
-    const u32 n = (ce > cb && !fix_now) ? (u32)(ce - cb) : 0u;
+    u32 n = (ce > cb && !fix_now) ? (u32)(ce - cb) : 0u;
+    if (lane == 0) a.edges += n;
+    const u64 lim = weight_limit(dh, minD);
+    const u32 wtop = (u32)umin64(lim - 1, kFull);
+    if (lim == 0) n = 0;
     run_pipeline(
         (n + kB - 1) / kB,
         [&](u32 b, u32 s) { issue_range_adj(st, s, d.in_adj, cb + b * kB, ce, lane); },
         [&](u32 b, u32 as, u32 ds) {
-            issue_dc<MULTI, L>(P, st, as, ds, min(kB, n - b * kB), cur, d.base, false, lane);
+            issue_nbr<MULTI, L>(P, st, as, ds, min(kB, n - b * kB), cur, d.base, wtop, false, lane);
         },
         [&](u32 b, u32 as, u32 ds) {
             const u32 nb = min(kB, n - b * kB);
 #pragma unroll
             for (u32 i = 0; i < kBI; ++i) {
                 const u32 sidx = 32 * i + lane;
-                if (sidx < nb) tv = min(tv, L::term(P, st.dc[ds][sidx], cur, st.adj[as][sidx].y, bd));
+                const u32 w = sidx < nb ? st.adj[as][sidx].y : 0u;
+                if (w) tv = min(tv, L::term(P, st.dc[ds][sidx], cur, w, bd));
             }
         });
     const u64 val = warp_min64((u64)tv);
     if (lane != 0) return;
-    a.edges += n;
     atomicMin(&P.L.hubmin[lo], val);
     // The arrival count is an acquire-release atomic: it publishes this
     // chunk's minimum and, for the last arrival, makes every other chunk's
@@ -1253,7 +1301,7 @@ __device__ void cup_hub(const RoundParams& P, InstCache<typename L::Term>* ic, W
                  : "memory");
     if (arrived != (nch << ps) - 1) return;
     // Last part of this hub's last chunk: finish the vertex.
-    const u64 m = atomicExch(&P.L.hubmin[lo], kInf64);
+    const u64 m = umin64(atomicExch(&P.L.hubmin[lo], kInf64), dh);
     P.L.hubcnt[lo] = 0;
     typename L::Rec* ry = L::rec(P) + g;
     const ulonglong2 v = L::ld_dc(ry, cur);
