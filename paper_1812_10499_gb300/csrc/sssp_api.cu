@@ -486,6 +486,8 @@ int init_single_context(sssp_graph* h) {
     P.g.base = 0;
     P.g.n = h->n;
     P.g.source = 0;
+    P.g.vd = h->vd;
+    P.g.wshift = h->wshift;
     c.narrow = h->narrow;
     if (c.narrow) {
         // Compact records, then (label-setting rounds, records held in L2)
@@ -681,49 +683,63 @@ int create_impl(sssp_graph* h, u32 n, u64 m, const u64* row_ptr, const u32* col,
     }
     h->n = n;
     h->m = m;
+    // Scratch of this setup, released when the stream has finished with it.
+    Pool tmp;
+    tmp.al = gp.al;
+    u32* cnt = nullptr;
+    int rc = SSSP_OK;
     if (csc_given) {
         CK(cudaMemcpyAsync(h->in_off, col_ptr, sizeof(u64) * ((size_t)n + 1),
                            cudaMemcpyHostToDevice, h->stream));
         RC(upload_adj(h, row, w_in, m, h->in_adj));
     } else {
-        // K0: transpose on the device (histogram, exclusive scan, scatter).
-        Pool tmp;
-        tmp.al = gp.al;
-        u64 *cnt = nullptr, *cursor = nullptr, *sums = nullptr;
-        const u64 cntn = (u64)n + 1;
-        int rc = tmp.get(&cnt, cntn);
-        if (rc == SSSP_OK) rc = tmp.get(&cursor, cntn);
+        // K0: transpose on the device (histogram, exclusive scan, scatter), the
+        // in-edges of a vertex in order of weight class.  (In-edges that the
+        // caller gives stay as they are.)
+        u64 *deg = nullptr, *sums = nullptr;
+        u32* cursor = nullptr;
+        const u64 cntn = (u64)n + 1, ncls = (u64)kClasses * n;
+        h->wshift = h->wmax >> 4 ? bits_for(h->wmax) - 4 : 0;
+        rc = tmp.get(&cnt, ncls);
+        if (rc == SSSP_OK) rc = tmp.get(&deg, cntn);
+        if (rc == SSSP_OK) rc = tmp.get(&cursor, ncls);
         if (rc == SSSP_OK) rc = tmp.get(&sums, (cntn + kScanTile - 1) / kScanTile + 1);
         cudaError_t e = cudaSuccess;
         if (rc == SSSP_OK) {
-            e = cudaMemsetAsync(cnt, 0, sizeof(u64) * cntn, h->stream);
+            e = cudaMemsetAsync(cnt, 0, sizeof(u32) * ncls, h->stream);
+            if (e == cudaSuccess) e = cudaMemsetAsync(deg + n, 0, sizeof(u64), h->stream);
             if (e == cudaSuccess && m) {
-                k_count_in<<<h->grid, kThreads, 0, h->stream>>>(h->out_adj, m, cnt);
+                k_count_in<<<h->grid, kThreads, 0, h->stream>>>(h->out_adj, m, h->wshift, cnt);
                 e = cudaGetLastError();
             }
-            if (e == cudaSuccess) rc = scan_excl(cnt, cntn, h->in_off, sums, h->stream);
-            if (rc == SSSP_OK && e == cudaSuccess)
-                e = cudaMemcpyAsync(cursor, h->in_off, sizeof(u64) * cntn, cudaMemcpyDeviceToDevice,
-                                    h->stream);
+            if (e == cudaSuccess) {
+                k_class_sums<<<h->grid, kThreads, 0, h->stream>>>(cnt, n, cursor, deg);
+                e = cudaGetLastError();
+            }
+            if (e == cudaSuccess) rc = scan_excl(deg, cntn, h->in_off, sums, h->stream);
             if (rc == SSSP_OK && e == cudaSuccess && m) {
-                k_scatter_in<<<h->grid, kThreads, 0, h->stream>>>(h->out_off, h->out_adj, n, cursor,
+                k_scatter_in<<<h->grid, kThreads, 0, h->stream>>>(h->out_off, h->out_adj, n,
+                                                                  h->wshift, h->in_off, cursor,
                                                                   h->in_adj);
                 e = cudaGetLastError();
             }
-            if (e == cudaSuccess) e = cudaStreamSynchronize(h->stream);
         }
-        tmp.release();
-        if (e != cudaSuccess) {
-            (void)cudaGetLastError();
-            return SSSP_E_CUDA;
-        }
-        RC(rc);
+        if (rc == SSSP_OK && e != cudaSuccess) rc = SSSP_E_CUDA;
     }
-    k_outw<<<h->grid, kThreads, 0, h->stream>>>(h->out_off, h->out_adj, n, h->outw);
-    CK(cudaGetLastError());
-    RC(gp.get(&h->inw, n));   // inWeight: the same reduction over the in-edges
-    k_outw<<<h->grid, kThreads, 0, h->stream>>>(h->in_off, h->in_adj, n, h->inw);
-    CK(cudaGetLastError());
+    if (rc == SSSP_OK) rc = gp.get(&h->inw, n);
+    if (rc == SSSP_OK) rc = gp.get(&h->vd, n);
+    if (rc == SSSP_OK) {
+        k_outw<<<h->grid, kThreads, 0, h->stream>>>(h->out_off, h->out_adj, n, h->outw);
+        // inWeight: the same reduction over the in-edges
+        k_outw<<<h->grid, kThreads, 0, h->stream>>>(h->in_off, h->in_adj, n, h->inw);
+        k_vdesc<<<h->grid, kThreads, 0, h->stream>>>(h->out_off, h->in_off, h->outw, h->inw, cnt, n,
+                                                     h->vd);
+        if (cudaGetLastError() != cudaSuccess) rc = SSSP_E_CUDA;
+    }
+    if (cudaStreamSynchronize(h->stream) != cudaSuccess && rc == SSSP_OK) rc = SSSP_E_CUDA;
+    tmp.release();
+    if (rc == SSSP_E_CUDA) (void)cudaGetLastError();
+    RC(rc);
     // The graph's degree statistics (its class in the tuning cache), then
     // the state that depends on the tuning.
     RC(count_hubs(h, h->opt.hub_degree, &h->hubs_out, &h->hubs_in, &h->max_out, &h->max_in));
@@ -993,13 +1009,14 @@ int batch_impl(const sssp_handle* g, const u32* sources, u32 k, u64* const* dist
                : nullptr;
     if (!c.exec) set_l2_window(c, h0->device);   // baked into the loop graph built next
     P.g = InstDesc{g[0]->out_off, g[0]->out_adj, g[0]->in_off, g[0]->in_adj,
-                   narrow ? g[0]->outw_pack : g[0]->outw, g[0]->inw, 0, g[0]->n, sources[0]};
+                   narrow ? g[0]->outw_pack : g[0]->outw, g[0]->inw, 0, g[0]->n, sources[0],
+                   g[0]->vd, g[0]->wshift};
     u64 page = 0;
     for (u32 i = 0; i < k; ++i) {
         const sssp_graph* gi = g[i];
         c.h_desc[i] = InstDesc{gi->out_off, gi->out_adj, gi->in_off, gi->in_adj,
                                narrow ? gi->outw_pack : gi->outw, gi->inw, page << kPageShift,
-                               gi->n, sources[i]};
+                               gi->n, sources[i], gi->vd, gi->wshift};
         const u64 np = ((u64)gi->n + (1u << kPageShift) - 1) >> kPageShift;
         for (u64 p = 0; p < np; ++p) c.h_pages[page + p] = i;
         page += np;

@@ -47,6 +47,32 @@ constexpr u32 kFixedN = 1u << 31;
 constexpr u64 kNarrowLimit = kFixedN - 1;   // distances must stay below this
 constexpr u32 kRelaxUnseen = 0x7FFFFFFFu;   // relaxation bound of an undiscovered vertex
 
+// In-edges are kept in order of weight class, so that a lower-bound scan which
+// needs only the light ones (weight_limit) reads a prefix of the row.  Eight
+// classes, finer at the light end, where most limits lie: in sixteenths of the
+// weight range (rounded up to a power of two), four of one, two of two, two of four.
+// With whole rows read, R-MAT 22 takes 2.65 ms where it now takes 2.09, R-MAT 18 with
+// wide records 2.16 (1.77), 64 sources on R-MAT 18 14.9 (12.5).
+constexpr u32 kClasses = 8;
+__host__ __device__ __forceinline__ u32 wclass(u32 w, u32 shift) {
+    const u32 t = (w >> shift) < 15 ? (w >> shift) : 15;
+    return t < 4 ? t : t < 8 ? 2 + (t >> 1) : 4 + (t >> 2);
+}
+
+// What a lower-bound step reads of a vertex's place in the graph: one 32-byte
+// sector in the place of four or five (offsets and weights in arrays of their
+// own), which in graphs of small degree were half of the step's memory traffic:
+// 128 random graphs of 4-16 edges per vertex 15.1 -> 12.1 ms, where the class counts
+// in an array of their own, a sector more, had cost as much as they saved.
+struct __align__(32) VDesc {
+    u64 ib;                 // first in-edge
+    u32 deg, odeg;          // in-degree, out-degree
+    u32 outw, inw;          // least out- and in-weight (kNoOutW: none)
+    u32 cum[2];             // byte k: the in-edges in weight classes 0 to k; above 255
+                            // in-edges, in 255ths of them, rounded up
+};
+static_assert(sizeof(VDesc) == 32, "VDesc must be one 32-byte sector");
+
 // Read-only description of one query's graph.
 struct InstDesc {
     const u64* out_off;     // CSR offsets, n + 1
@@ -58,6 +84,9 @@ struct InstDesc {
     u64 base;               // global record index of local vertex 0
     u32 n;
     u32 source;
+    const VDesc* vd;        // per vertex, or nullptr (the arrays above are read instead,
+                            // and whole rows of in-edges)
+    u32 wshift;             // of the weight classes
 };
 
 enum : u32 { kIdle = 0, kRunning = 1, kDone = 2, kStopped = 3, kErrRounds = 4 };

@@ -52,9 +52,12 @@ __global__ void k_finalize(const VRec* rec, const VRecN* recn, const int* frec, 
 __global__ void k_finalize_multi(RoundParams P, u64 nrec, u64* dist);
 __global__ void k_interleave(const u32* col, const u32* w, u64 m, uint2* adj);
 __global__ void k_find_loop(const u64* out_off, const uint2* out_adj, u32 n, u32* flag);
-__global__ void k_count_in(const uint2* adj, u64 m, u64* cnt);
-__global__ void k_scatter_in(const u64* out_off, const uint2* out_adj, u32 n, u64* cursor,
-                             uint2* in_adj);
+__global__ void k_count_in(const uint2* adj, u64 m, u32 wshift, u32* cnt);
+__global__ void k_class_sums(u32* cnt, u32 n, u32* cursor, u64* deg);
+__global__ void k_vdesc(const u64* out_off, const u64* in_off, const u32* outw, const u32* inw,
+                        const u32* sums, u32 n, VDesc* vd);
+__global__ void k_scatter_in(const u64* out_off, const uint2* out_adj, u32 n, u32 wshift,
+                             const u64* in_off, u32* cursor, uint2* in_adj);
 __global__ void k_outw(const u64* out_off, const uint2* out_adj, u32 n, u32* outw);
 __global__ void k_pack_outw(const u32* outw, const u64* in_off, u32 n, u32 hub, u32* out);
 __global__ void k_count_hubs(const u64* out_off, const u64* in_off, u32 n, u32 hub, u32* cnt);
@@ -238,6 +241,8 @@ struct sssp_graph {
     u32* outw = nullptr;
     u32* outw_pack = nullptr;        // compact layout: outWeight | in-hub flag (k_pack_outw)
     u32* inw = nullptr;              // inWeight: min in-edge weight (kNoOutW: none)
+    sssp::VDesc* vd = nullptr;       // per vertex (InstDesc::vd)
+    u32 wshift = 0;
     cudaStream_t stream = nullptr;   // internal stream for setup and host-pointer solves
     int grid = 0;
     int grid_solve = 0;

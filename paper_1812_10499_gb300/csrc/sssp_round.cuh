@@ -690,9 +690,43 @@ __device__ __forceinline__ void issue_dc(const RoundParams& P, WarpStage<S>& st,
 // edges with w < D[y] - minD, and D[y], is the minimum over all.
 __device__ __forceinline__ u64 weight_limit(u64 dy, u64 minD) { return dy > minD ? dy - minD : 0; }
 
+// The description of vertex v, loaded whole beside the vertex's state: the prefix
+// that the limit asks for costs no further round trip.  Without descriptions (the
+// caller's own arrays), from the graph's arrays.
+template <class L>
+__device__ __forceinline__ VDesc vertex_desc(const RoundParams& P, const InstDesc& d, u32 v,
+                                             const typename L::Rec* r) {
+    VDesc x;
+    if (d.vd) {
+        const uint4* p = reinterpret_cast<const uint4*>(d.vd + v);
+        const uint4 a = __ldg(p), b = __ldg(p + 1);
+        x.ib = a.x | (u64)a.y << 32;
+        x.deg = a.z;
+        x.odeg = a.w;
+        x.outw = b.x;
+        x.inw = b.y;
+        x.cum[0] = b.z;
+        x.cum[1] = b.w;
+    } else {
+        x.ib = d.in_off[v];
+        x.deg = (u32)(d.in_off[v + 1] - x.ib);
+        x.odeg = (u32)(d.out_off[v + 1] - d.out_off[v]);
+        x.outw = outw_of<L>(d, r, v);
+        x.inw = P.cheap ? d.inw[v] : 0u;
+        x.cum[0] = x.cum[1] = kFull;
+    }
+    return x;
+}
+// At least the in-edges with weights up to wtop, from the start of the row.
+__device__ __forceinline__ u32 light_prefix(const VDesc& x, u32 wtop, u32 shift) {
+    const u32 k = wclass(wtop, shift);
+    const u32 b = ((k & 4 ? x.cum[1] : x.cum[0]) >> (8 * (k & 3))) & 255u;
+    return x.deg <= 255 ? min(b, x.deg) : (u32)(((u64)b * x.deg + 254) / 255);
+}
+
 // Starts gathering the source states of the nb in-edges in adjacency slot as
 // into state slot ds, of those edges whose weight is at most the owner's wtop;
-// the others get weight 0 (no edge has it) and are passed over.  The gathers are
+// the others get source kFull (no vertex has it) and are passed over.  The gathers are
 // what a large lower-bound phase waits on: 32 bytes of L2 per edge at random,
 // beside 8 bytes of adjacency in sequence.  On R-MAT 22 (weights to 255) 10-25%
 // of the in-edges are kept, 2.79 -> 2.65 ms a solve; on 128 random graphs (to
@@ -717,7 +751,7 @@ __device__ __forceinline__ void issue_nbr(const RoundParams& P, WarpStage<S>& st
         if (!ev) continue;
         const uint2 e = st.adj[as][idx];
         if (e.y <= top) st.dc[ds][idx].issue(rec + (u32)(ob + e.x), cur);
-        else st.adj[as][idx].y = 0u;
+        else st.adj[as][idx].x = kFull;
     }
 }
 
@@ -1076,9 +1110,10 @@ __device__ __forceinline__ T seg_min(T v, u32 brk, u32 lane) {
 // The cheaper fixing rules tried before the in-edge scan: SP_2's in-version
 // rule D[y] <= minD + inWeight[y] (Sec. IV) and D[y] <= threshold (Lemma 8).
 // Each implies that Eq. (1) gives C[y] = D[y]: a fixed in-neighbour x gives
-// D[x] + w >= D[y], an unfixed one lb(x) + w >= minD + inWeight[y].
+// D[x] + w >= D[y], an unfixed one lb(x) + w >= minD + inWeight[y].  (An active
+// vertex has an in-edge, so its inWeight is a weight, also when it is 2^32 - 1.)
 __device__ __forceinline__ bool cheap_rules_fix(u64 dy, u32 inw, u64 thr, u64 minD) {
-    return (inw != kNoOutW && dy <= minD + inw) || dy <= thr;
+    return dy <= minD + inw || dy <= thr;
 }
 
 // Windowed relaxation: the bound below which a changed active vertex relaxes
@@ -1111,9 +1146,10 @@ __device__ void cup_small(const RoundParams& P, InstCache<typename L::Term>* ic,
     const u32 nxt = cur ^ 1u;
     const u32 idx = (t << ts) + lane;
     const bool valid = (lane >> ts) == 0 && idx < nas;
-    u32 g = 0, yloc = 0, inst = 0, deg = 0, outw = kNoOutW;
-    u64 gbase = 0, ib = 0, dy = 0, cy = 0, thr = thr0, minD = minD0, odeg = 0;
+    u32 g = 0, yloc = 0, inst = 0, deg = 0, wshift = 0;
+    u64 gbase = 0, dy = 0, cy = 0, thr = thr0, minD = minD0;
     bool fix_now = false;
+    VDesc x = {0, 0, 0, kNoOutW, kNoOutW, {0, 0}};
     const uint2* in_adj = P.g.in_adj;
     typename L::Rec* rec = L::rec(P);
     if (valid) {
@@ -1126,15 +1162,14 @@ __device__ void cup_small(const RoundParams& P, InstCache<typename L::Term>* ic,
             minD = P.ivar[inst].minD[cur];
         }
         yloc = g - (u32)gbase;
-        ib = d.in_off[yloc];
-        deg = (u32)(d.in_off[yloc + 1] - ib);
-        // Out-degree now, in the same round trip (needed if y gets fixed).
-        odeg = d.out_off[yloc + 1] - d.out_off[yloc];
+        // (One round trip: the out-degree is needed if y gets fixed.)
+        x = vertex_desc<L>(P, d, yloc, rec + g);
+        wshift = d.wshift;
         const ulonglong2 v = L::ld_dc(rec + g, cur);
         dy = v.x >> P.vbits;
         cy = v.y & kCMask;
-        outw = outw_of<L>(d, rec + g, yloc);
-        if (P.cheap) fix_now = cheap_rules_fix(dy, d.inw[yloc], thr, minD);
+        deg = x.deg;
+        if (P.cheap) fix_now = cheap_rules_fix(dy, x.inw, thr, minD);
         // SP_1: every in-edge relaxed by a fixed source, so D[y] is final.
         if (L::kPred && !fix_now) fix_now = P.pcnt[g] == 0u;
         if (fix_now) deg = 0;                     // its in-edges are not read
@@ -1143,6 +1178,7 @@ __device__ void cup_small(const RoundParams& P, InstCache<typename L::Term>* ic,
     const u64 lim = weight_limit(dy, minD);
     const u32 wtop = (u32)umin64(lim - 1, kFull);
     if (lim == 0) deg = 0;                        // none of its in-edges can matter
+    else if (deg) deg = light_prefix(x, wtop, wshift);
     // The owners' minima: 64-bit slots, or (compact layout, SHATOM) 32-bit
     // slots in their place.
     constexpr bool kAtom = SHATOM && L::kNarrow;
@@ -1150,7 +1186,7 @@ __device__ void cup_small(const RoundParams& P, InstCache<typename L::Term>* ic,
     if (kAtom) smin32[lane] = (u32)dy;
     else smin[lane] = dy;
     const typename L::Bounds bd = L::bounds(thr, minD);
-    Tile tl = make_tile(st, deg, (u64)(in_adj + ib), lane);
+    Tile tl = make_tile(st, deg, (u64)(in_adj + x.ib), lane);
     run_pipeline(
         (tl.total + kB - 1) / kB,
         [&](u32 b, u32 s) { issue_tile_adj(st, tl, s, b * kB, deg, lane); },
@@ -1172,13 +1208,14 @@ __device__ void cup_small(const RoundParams& P, InstCache<typename L::Term>* ic,
                     ob.minD = __shfl_sync(kFull, bd.minD, own);
                 }
                 typename L::Term val = L::kTermInf;
-                const u32 w = ev ? st.adj[as][sidx].y : 0u;
-                if (w) val = L::term(P, st.dc[ds][sidx], cur, w, ob);
+                const uint2 e = ev ? st.adj[as][sidx] : make_uint2(kFull, 0u);
+                const bool on = e.x != kFull;
+                if (on) val = L::term(P, st.dc[ds][sidx], cur, e.y, ob);
                 if (kAtom) {
-                    if (w) atomicMin(smin32 + own, (u32)val);
+                    if (on) atomicMin(smin32 + own, (u32)val);
                     continue;
                 }
-                if (!__any_sync(kFull, w != 0)) continue;
+                if (!__any_sync(kFull, on)) continue;
                 // Min over the lanes sharing an owner (contiguous lanes; a
                 // segment starts at every owner change).
                 const u32 prev = __shfl_up_sync(kFull, own, 1);
@@ -1224,12 +1261,12 @@ __device__ void cup_small(const RoundParams& P, InstCache<typename L::Term>* ic,
         }
         warp_append(P, &P.ctl->nFX[nxt], P.L.FX[nxt], valid && fix, g, lane);
     }
-    const bool fs = fx && odeg <= P.hub;
+    const bool fs = fx && x.odeg <= P.hub;
     if (P.lc) wq_push(P, qf, &P.ctl->nFX[nxt], P.L.FX[nxt], valid && fix, g, lane);
     else wq_push(P, qf, &P.ctl->nFS[nxt], P.L.FS[nxt], fs, g, lane);
-    if (fx && !fs) put_hub(P, &P.ctl->FHpk[nxt], P.L.FH[nxt], P.L.FC[nxt], g, odeg);
+    if (fx && !fs) put_hub(P, &P.ctl->FHpk[nxt], P.L.FH[nxt], P.L.FC[nxt], g, x.odeg);
     wq_push(P, qa, &P.ctl->nAS[nxt], P.L.AS[nxt], sv, g, lane);
-    const u64 tsum = outw == kNoOutW ? P.dinf : dy + outw;
+    const u64 tsum = x.outw == kNoOutW ? P.dinf : dy + x.outw;
     if (MULTI) {
         if (fx) inst_count(P, ic, inst, nxt);
         if (sv) inst_fold(P, ic, inst, nxt, dy, tsum);
@@ -1256,8 +1293,9 @@ __device__ void cup_hub(const RoundParams& P, InstCache<typename L::Term>* ic, W
         minD = P.ivar[inst].minD[cur];
     }
     const u32 yloc = g - (u32)d.base;
-    const u64 ib = d.in_off[yloc], ie = d.in_off[yloc + 1];
-    const u32 nch = (u32)((ie - ib + P.chunk - 1) / P.chunk);   // as counted by put_hub
+    const VDesc x = vertex_desc<L>(P, d, yloc, L::rec(P) + g);
+    const u64 ib = x.ib, ie = ib + x.deg;
+    const u32 nch = (u32)(((u64)x.deg + P.chunk - 1) / P.chunk);   // as counted by put_hub
     const u64 cb = ib + (u64)k * P.chunk + ((P.chunk * part) >> ps);
     const u64 ce = umin64(ib + (u64)k * P.chunk + ((P.chunk * (part + 1)) >> ps), ie);
     const typename L::Bounds bd = L::bounds(thr, minD);
@@ -1266,16 +1304,21 @@ __device__ void cup_hub(const RoundParams& P, InstCache<typename L::Term>* ic, W
     // predecessor counts do not change during this phase).
     bool fix_now = false;
     const u64 dh = L::ld_dc(L::rec(P) + g, cur).x >> P.vbits;
-    if (P.cheap) fix_now = cheap_rules_fix(dh, d.inw[yloc], thr, minD);
+    if (P.cheap) fix_now = cheap_rules_fix(dh, x.inw, thr, minD);
     if (L::kPred && !fix_now) fix_now = P.pcnt[g] == 0u;
     u32 n = (ce > cb && !fix_now) ? (u32)(ce - cb) : 0u;
     if (lane == 0) a.edges += n;
     const u64 lim = weight_limit(dh, minD);
     const u32 wtop = (u32)umin64(lim - 1, kFull);
-    if (lim == 0) n = 0;
+    if (lim == 0) {
+        n = 0;
+    } else if (n) {
+        const u64 end = ib + light_prefix(x, wtop, d.wshift);
+        n = end > cb ? (u32)umin64(n, end - cb) : 0u;
+    }
     run_pipeline(
         (n + kB - 1) / kB,
-        [&](u32 b, u32 s) { issue_range_adj(st, s, d.in_adj, cb + b * kB, ce, lane); },
+        [&](u32 b, u32 s) { issue_range_adj(st, s, d.in_adj, cb + b * kB, cb + n, lane); },
         [&](u32 b, u32 as, u32 ds) {
             issue_nbr<MULTI, L>(P, st, as, ds, min(kB, n - b * kB), cur, d.base, wtop, false, lane);
         },
@@ -1284,13 +1327,14 @@ __device__ void cup_hub(const RoundParams& P, InstCache<typename L::Term>* ic, W
 #pragma unroll
             for (u32 i = 0; i < kBI; ++i) {
                 const u32 sidx = 32 * i + lane;
-                const u32 w = sidx < nb ? st.adj[as][sidx].y : 0u;
-                if (w) tv = min(tv, L::term(P, st.dc[ds][sidx], cur, w, bd));
+                if (sidx >= nb) continue;
+                const uint2 e = st.adj[as][sidx];
+                if (e.x != kFull) tv = min(tv, L::term(P, st.dc[ds][sidx], cur, e.y, bd));
             }
         });
     const u64 val = warp_min64((u64)tv);
     if (lane != 0) return;
-    atomicMin(&P.L.hubmin[lo], val);
+    if (n) atomicMin(&P.L.hubmin[lo], val);
     // The arrival count is an acquire-release atomic: it publishes this
     // chunk's minimum and, for the last arrival, makes every other chunk's
     // minimum visible before the vertex is finished.
@@ -1307,7 +1351,6 @@ __device__ void cup_hub(const RoundParams& P, InstCache<typename L::Term>* ic, W
     const ulonglong2 v = L::ld_dc(ry, cur);
     const u64 dy = v.x >> P.vbits;
     const u64 cy = v.y & kCMask;
-    const u32 outw = outw_of<L>(d, ry, yloc);
     bool fix = true;
     u64 cn = dy;
     if (!fix_now) cn = decide(P, dy, cy, m, thr, minD, fix);
@@ -1321,7 +1364,7 @@ __device__ void cup_hub(const RoundParams& P, InstCache<typename L::Term>* ic, W
         if (P.lc || P.win) put_small(P, P.L.FX[nxt], atomicAdd(&P.ctl->nFX[nxt], 1u), g);
     } else {
         put_hub(P, &P.ctl->AHpk[nxt], P.L.AH[nxt], P.L.AC[nxt], g, ie - ib);
-        const u64 t = outw == kNoOutW ? P.dinf : dy + outw;
+        const u64 t = x.outw == kNoOutW ? P.dinf : dy + x.outw;
         if (MULTI) inst_fold(P, ic, inst, nxt, dy, t);
         else fold(dy, t, an);
     }
@@ -1333,9 +1376,8 @@ __device__ void cup_hub(const RoundParams& P, InstCache<typename L::Term>* ic, W
         }
     }
     if (front) {
-        const u64 odeg = d.out_off[yloc + 1] - d.out_off[yloc];
-        if (odeg <= P.hub) put_small(P, P.L.FS[nxt], atomicAdd(&P.ctl->nFS[nxt], 1u), g);
-        else put_hub(P, &P.ctl->FHpk[nxt], P.L.FH[nxt], P.L.FC[nxt], g, odeg);
+        if (x.odeg <= P.hub) put_small(P, P.L.FS[nxt], atomicAdd(&P.ctl->nFS[nxt], 1u), g);
+        else put_hub(P, &P.ctl->FHpk[nxt], P.L.FH[nxt], P.L.FC[nxt], g, x.odeg);
         if (MULTI) inst_count(P, ic, inst, nxt);
         else an.nfix++;
     }

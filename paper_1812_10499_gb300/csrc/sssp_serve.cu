@@ -218,7 +218,8 @@ int admit(sssp_server* s, u64 step) {
         const sssp_graph* g = q->g;
         c.h_desc[slot] = InstDesc{g->out_off, g->out_adj, g->in_off, g->in_adj,
                                   s->narrow ? g->outw_pack : g->outw, g->inw,
-                                  (u64)first << kPageShift, g->n, q->source};
+                                  (u64)first << kPageShift, g->n, q->source, g->vd,
+                                  g->wshift};
         CK(cudaMemcpyAsync((void*)(c.P.idesc + slot), c.h_desc + slot, sizeof(InstDesc),
                            cudaMemcpyHostToDevice, s->stream));
         CK(cudaMemcpyAsync((void*)(c.P.page_owner + first), c.h_pages + first,

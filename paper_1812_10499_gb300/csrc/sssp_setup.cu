@@ -150,22 +150,72 @@ __global__ void k_find_loop(const u64* out_off, const uint2* out_adj, u32 n, u32
     }
 }
 
-__global__ void k_count_in(const uint2* adj, u64 m, u64* cnt) {
+// In-edges of every vertex by weight class.
+__global__ void k_count_in(const uint2* adj, u64 m, u32 wshift, u32* cnt) {
     for (u64 i = blockIdx.x * (u64)blockDim.x + threadIdx.x; i < m;
-         i += (u64)gridDim.x * blockDim.x)
-        atomicAdd(&cnt[adj[i].x], 1ull);
+         i += (u64)gridDim.x * blockDim.x) {
+        const uint2 e = adj[i];
+        atomicAdd(&cnt[(u64)kClasses * e.x + wclass(e.y, wshift)], 1u);
+    }
 }
 
-// One warp per source vertex scatters its out-edges into the in-lists.
-__global__ void k_scatter_in(const u64* out_off, const uint2* out_adj, u32 n, u64* cursor,
-                             uint2* in_adj) {
+// The class counts of every vertex: to sums up to and with each class (in
+// place), to sums before it (cursor), and their total (deg).
+__global__ void k_class_sums(u32* cnt, u32 n, u32* cursor, u64* deg) {
+    static_assert(kClasses == 8, "two 16-byte words per vertex");
+    for (u64 v = blockIdx.x * (u64)blockDim.x + threadIdx.x; v < n;
+         v += (u64)gridDim.x * blockDim.x) {
+        uint4* c = reinterpret_cast<uint4*>(cnt) + 2 * v;
+        uint4* b = reinterpret_cast<uint4*>(cursor) + 2 * v;
+        uint4 x = c[0], y = c[1];
+        x.y += x.x;
+        x.z += x.y;
+        x.w += x.z;
+        y.x += x.w;
+        y.y += y.x;
+        y.z += y.y;
+        y.w += y.z;
+        c[0] = x;
+        c[1] = y;
+        b[0] = make_uint4(0u, x.x, x.y, x.z);
+        b[1] = make_uint4(x.w, y.x, y.y, y.z);
+        deg[v] = y.w;
+    }
+}
+
+// The vertices' descriptions; sums: the in-edges by weight class (k_class_sums), or
+// nullptr when the rows are in no such order (every prefix is the whole row then).
+__global__ void k_vdesc(const u64* out_off, const u64* in_off, const u32* outw, const u32* inw,
+                        const u32* sums, u32 n, VDesc* vd) {
+    for (u64 v = blockIdx.x * (u64)blockDim.x + threadIdx.x; v < n;
+         v += (u64)gridDim.x * blockDim.x) {
+        VDesc d;
+        d.ib = in_off[v];
+        d.deg = (u32)(in_off[v + 1] - d.ib);
+        d.odeg = (u32)(out_off[v + 1] - out_off[v]);
+        d.outw = outw[v];
+        d.inw = inw[v];
+        d.cum[0] = d.cum[1] = 0;
+        for (u32 k = 0; k < kClasses; ++k) {
+            const u32 c = sums ? sums[kClasses * v + k] : d.deg;
+            const u32 b = d.deg <= 255 ? c : (u32)(((u64)c * 255 + d.deg - 1) / d.deg);
+            d.cum[k >> 2] |= b << (8 * (k & 3));
+        }
+        vd[v] = d;
+    }
+}
+
+// One warp per source vertex scatters its out-edges into the in-lists, each into
+// its weight class.
+__global__ void k_scatter_in(const u64* out_off, const uint2* out_adj, u32 n, u32 wshift,
+                             const u64* in_off, u32* cursor, uint2* in_adj) {
     const u32 lane = threadIdx.x & 31u;
     for (u64 u = (blockIdx.x * (u64)blockDim.x + threadIdx.x) >> 5; u < n;
          u += ((u64)gridDim.x * blockDim.x) >> 5) {
         for (u64 k = out_off[u] + lane; k < out_off[u + 1]; k += 32) {
             const uint2 e = out_adj[k];
-            const u64 pos = atomicAdd(&cursor[e.x], 1ull);
-            in_adj[pos] = make_uint2((u32)u, e.y);
+            const u32 at = atomicAdd(&cursor[(u64)kClasses * e.x + wclass(e.y, wshift)], 1u);
+            in_adj[in_off[e.x] + at] = make_uint2((u32)u, e.y);
         }
     }
 }

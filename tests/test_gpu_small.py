@@ -107,3 +107,54 @@ def test_self_loops_are_dropped(sssp_lib, given_csc, where):
         sssp_lib.sssp_destroy(h)
     ref = oracle.round_r(base, 5)
     assert np.array_equal(out["dist"], ref.dist) and np.array_equal(out["parent"], ref.parent)
+
+
+WEIGHTS = {"unit": [1], "pair": [1, 2], "fifteen": list(range(1, 17)), "steps": [15, 16, 17, 31, 32, 33],
+           "range": list(range(1, 256)), "spread": [1, 1000, 1 << 20], "top": [1, 1 << 31, 0xFFFFFFFF]}
+
+
+@LAYOUTS
+@pytest.mark.parametrize("given_csc", [False, True])
+@pytest.mark.parametrize("mode,delta", [(oracle.RULE_THR, None), (oracle.RULE_MIND, None),
+                                        (oracle.CHEAP_FIRST, None), (oracle.LABEL_CORRECT, None),
+                                        (oracle.RULE_THR, 40)],
+                         ids=["threshold", "mind", "cheap", "correcting", "windowed"])
+@pytest.mark.parametrize("weights", list(WEIGHTS))
+def test_in_edges_by_weight_class(sssp_lib, layout, given_csc, mode, delta, weights):
+    """The lower bounds of the full-grid kernels, over rows in order of weight class
+    and (the caller's CSC) over rows in any order: weights at the edges of the
+    classes, rows of no in-edge up to several hub chunks, both round drivers."""
+    P, n = sssp_lib, 2500
+    g = gg.random_var_graph(n, 0, 9, 1, 50, 21)
+    src, col, _ = g.edges()
+    extra = np.arange(1, n, dtype=np.uint32)
+    src = np.concatenate([src, extra, np.zeros(40, np.uint32)])
+    col = np.concatenate([col, np.where(extra == 7, 8, 7).astype(np.uint32),   # a hub at 7
+                          np.arange(1, 41, dtype=np.uint32)])
+    pick = gg.uniform(9, 2, len(src), 0, len(WEIGHTS[weights]) - 1)
+    w = np.array(WEIGHTS[weights], dtype=np.uint32)[pick.astype(np.int64)]
+    g = gg.from_edges(n, list(zip(src.tolist(), col.tolist(), w.tolist())))
+    csc = {}
+    if given_csc:
+        s, c, ww = g.edges()
+        order = np.argsort(c, kind="stable")[::-1]
+        order = order[np.argsort(c[order], kind="stable")]
+        ptr = np.concatenate([[0], np.cumsum(np.bincount(c, minlength=n))])
+        csc = dict(col_ptr=ptr.astype(np.uint64), row=s[order], w_in=ww[order])
+    ref = oracle.round_r(g, 0, mode=mode, delta=delta)
+    for loop in (P.SSSP_LOOP_HOST, P.SSSP_LOOP_GRAPH):
+        opt = P.sssp_options_default()
+        opt.layout = layout if n * max(WEIGHTS[weights]) < 2**31 - 1 else P.SSSP_LAYOUT_WIDE
+        opt.loop_mode, opt.rule = loop, mode
+        opt.hub_degree, opt.chunk_edges = 64, 512
+        if delta is not None:
+            opt.rule, opt.delta = P.SSSP_RULE_WINDOWED, delta
+        h = P.sssp_create(g.n, g.row_ptr, g.col, g.w, options=opt, **csc)
+        try:
+            out = P.sssp_solve_ex(h, 0, parent=True, fixed_round=True, lower=True)
+        finally:
+            P.sssp_destroy(h)
+        assert np.array_equal(out["dist"], ref.dist) and np.array_equal(out["parent"], ref.parent)
+        assert np.array_equal(out["fixed_round"], ref.fixed_round)
+        assert np.array_equal(out["lower"], ref.C)
+        assert out["info"]["in_scanned"] == ref.stats["in_scanned"]
