@@ -548,7 +548,8 @@ def run_ours(args):
         timing = ("CUDA events around every launch on the solve stream; the host launches the "
                   "device loop's iterations (k_relax, k_cupdate, cluster tail kernel k_tail) as "
                   "the timed solves run them; algorithmic bytes from the work counters of the "
-                  "rounds each kernel ran")
+                  "rounds each kernel ran, with every in-edge of a scanned vertex counted, also "
+                  "those too heavy to matter, which k_cupdate does not read")
     dom_gbs = bytes_per_launch / (ms_per_launch * 1e-3) / 1e9
     traffic, traffic_src = measured_traffic(kernel, args.config, bytes_per_launch)
     # Whole step: all algorithmic bytes of the 8 solves over the timed step.

@@ -77,7 +77,7 @@ extern "C" {
  * y at once when D[y] <= minD + inWeight[y] (the in-version rule of SP_2,
  * Sec. IV, inWeight = least in-edge weight) or D[y] <= threshold (Lemma 8).
  * Both imply that Eq. (1) gives C[y] = D[y], so every output is unchanged;
- * only in_scanned (the in-edges actually read) drops. */
+ * only in_scanned drops (the in-edges of the vertices that are scanned). */
 #define SSSP_RULE_CHEAP_FIRST 4u
 /* Flag OR-ed into the rule: windowed relaxation, a combination of the lower
  * bounds with Delta-stepping (Sec. I notes that the two can be combined).
@@ -304,7 +304,8 @@ typedef struct sssp_solve_info {
                                 a target                                                   */
     uint64_t reached;        /* vertices fixed (reachable, source included)                */
     uint64_t out_scanned;    /* out-edges scanned by step (a)                              */
-    uint64_t in_scanned;     /* in-edges scanned by step (b)                               */
+    uint64_t in_scanned;     /* in-edges of the vertices scanned by step (b); of those, the
+                                ones too heavy to lower the minimum are not read           */
     uint64_t active_visits;  /* sum over rounds of the discovered-unfixed set size         */
     uint64_t front_visits;   /* sum over rounds of the frontier size                       */
     uint64_t kernel_launches;/* kernels the solve launched (start, rounds, output)          */
