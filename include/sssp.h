@@ -430,7 +430,8 @@ void sssp_serve_close(sssp_server* s);
  * the round kernels from the host and bracket every launch with CUDA events
  * on the solve stream.  With the default loop mode (SSSP_LOOP_GRAPH) the
  * host launches exactly the device loop's iterations -- k_relax, k_cupdate,
- * then the cluster tail kernel k_tail, which runs the following small rounds
+ * then the cluster kernel of the small rounds (k_small or k_tail; "tail" below),
+ * which runs the following small rounds
  * -- so the times describe the schedule of an unprofiled solve; with
  * SSSP_LOOP_HOST every iteration is one round of k_relax and k_cupdate.
  * Launches after the last round are not counted.  The work counters of
@@ -442,11 +443,11 @@ typedef struct sssp_kernel_profile {
     double relax_ms;         /* summed event time of k_relax launches    */
     double cupdate_ms;       /* summed event time of k_cupdate launches  */
     uint64_t tail_launches;
-    double tail_ms;          /* summed event time of k_tail launches     */
-    uint64_t tail_rounds;    /* rounds finished inside k_tail            */
+    double tail_ms;          /* summed event time of the cluster kernel's launches */
+    uint64_t tail_rounds;    /* rounds finished inside it                */
     uint64_t grid_counters[4];  /* out_scanned, in_scanned, active_visits, front_visits
                                    of the work done by k_relax and k_cupdate */
-    uint64_t tail_counters[4];  /* the same for the work done by k_tail   */
+    uint64_t tail_counters[4];  /* the same for the cluster kernel's work */
 } sssp_kernel_profile;
 
 /* enable: 1 = on, 0 = off.  out (nullable) receives the totals gathered
@@ -455,8 +456,8 @@ int sssp_profile(sssp_handle h, int enable, sssp_kernel_profile* out);
 
 /* Per-iteration event times of the most recent profiled solve (iterations
  * of the device loop, or rounds with SSSP_LOOP_HOST): iteration i's
- * k_relax / k_cupdate / k_tail milliseconds go to relax_ms[i] /
- * cupdate_ms[i] / tail_ms[i], the rounds k_tail finished to tail_rounds[i],
+ * k_relax / k_cupdate / cluster kernel milliseconds go to relax_ms[i] /
+ * cupdate_ms[i] / tail_ms[i], the rounds the latter finished to tail_rounds[i],
  * and (device-loop schedule only, else 0) the work counters of its k_relax
  * and k_cupdate -- out_scanned, in_scanned, active_visits, front_visits --
  * to grid_counters[4i .. 4i+3], for i < cap (tail_ms, tail_rounds and

@@ -25,8 +25,11 @@
 // load balance over their edges, or one chunk of a hub vertex.  Edges go
 // through a per-warp three-stage cp.async pipeline in shared memory:
 // adjacency two batches ahead, neighbour states one batch ahead, compute on
-// the current batch.  List appends go through warp-private buffers flushed
-// 32 entries per atomic.  Every kernel is templated on the state layout:
+// the current batch.  A lower-bound scan reads the in-edges light enough to
+// matter: a prefix of the row, which is in order of weight class (sssp_dev.cuh,
+// weight_limit).  List appends go through warp-private buffers of kQFlush
+// entries per atomic; what is left at a phase's end leaves with the CTA's minima
+// and counters, one atomic per word (end_phase).  Every kernel is templated on the state layout:
 // 32-byte records (WideL) or 16-byte records (NarrowL), either of them
 // with predecessor counts (PredL).
 #pragma once
@@ -349,7 +352,9 @@ __device__ __forceinline__ u32 static_item(u32 wib) {
 // batch by batch, and each batch waits for the one before; so when the lists
 // are too short to give every warp of the grid a full item, the items are made
 // smaller instead: list tiles of 2^ts entries (32 at most), hub chunks in 2^ps
-// parts of at least 128 edges.
+// parts of at least 128 edges.  R-MAT 18 with wide records 3.99 -> 2.58 ms, R-MAT 20
+// 1.73 -> 1.60, layered DAG 14.7 -> 13.7.  Cutting on to two or four items per warp
+// costs the DAG (10.6 ms by then) 2.3 and 4.7 ms: an item's start is its longest part.
 struct Split {
     u32 ts, ps;
     u32 tiles, parts;       // items of either kind
@@ -403,6 +408,7 @@ __device__ __forceinline__ void atomic_min_checked(u64* p, u64 v) {
 // the same few scalars: folded there one by one (a load and perhaps an atomic
 // each), 4 sources on R-MAT 18 took 2.5 times as long in the relaxation as one
 // query with the same work.  Slots beyond the cache fold in global memory.
+// Batch of 128 graphs 17.9 -> 14.9 ms, 64 sources on R-MAT 18 19.5 -> 17.5.
 constexpr u32 kInstCache = 1024;
 template <class D>
 struct InstCache {
@@ -463,6 +469,7 @@ __device__ __forceinline__ void fold(u64 d, u64 t, Acc& a) {
 // together, with one atomic per word and CTA (all threads of the CTA).  The
 // words are shared by the whole grid, and an atomic on one word takes about 4
 // cycles of its L2 slice: one per warp, from 3648 warps, would take 7 us a word.
+// (With the words 128 bytes apart: R-MAT 20 1.60 -> 1.42 ms, layered DAG 13.7 -> 11.6.)
 template <bool MULTI, bool NARROW, class D>
 __device__ __forceinline__ void end_phase(const RoundParams& P, InstCache<D>* ic, u32 slot,
                                           u32 nfix_slot, const Acc& a, u32 stat_edges, u32 stat_visits,
