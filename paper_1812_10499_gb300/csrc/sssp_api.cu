@@ -625,6 +625,79 @@ int upload_adj(sssp_graph* h, const u32* idx, const u32* w, u64 m, uint2* adj) {
     return rc;
 }
 
+// The device transposition (histogram, exclusive scan, scatter), the in-edges of a
+// vertex in order of weight class.  *sums: the in-edges of every vertex in classes 0
+// to k, from tmp.  The counts have 32 bits: when some vertex has more in-edges
+// (parallel edges, of a graph with more than 2^32 - 1), their total falls short of m
+// and *counted is false, with nothing placed.
+int transpose_by_class(sssp_graph* h, Pool& tmp, u32** sums, bool* counted) {
+    const u32 n = h->n;
+    const u64 m = h->m, cntn = (u64)n + 1, ncls = (u64)kClasses * n;
+    u32 *cnt = nullptr, *cursor = nullptr;
+    u64 *deg = nullptr, *scan = nullptr;
+    *counted = true;
+    h->wshift = h->wmax >> 4 ? bits_for(h->wmax) - 4 : 0;
+    RC(tmp.get(&cnt, ncls));
+    RC(tmp.get(&deg, cntn));
+    RC(tmp.get(&cursor, ncls));
+    RC(tmp.get(&scan, (cntn + kScanTile - 1) / kScanTile + 1));
+    CK(cudaMemsetAsync(cnt, 0, sizeof(u32) * ncls, h->stream));
+    CK(cudaMemsetAsync(deg + n, 0, sizeof(u64), h->stream));
+    if (m) {
+        k_count_in<<<h->grid, kThreads, 0, h->stream>>>(h->out_adj, m, h->wshift, cnt);
+        CK(cudaGetLastError());
+    }
+    k_class_sums<<<h->grid, kThreads, 0, h->stream>>>(cnt, n, cursor, deg);
+    CK(cudaGetLastError());
+    RC(scan_excl(deg, cntn, h->in_off, scan, h->stream));
+    if (m > kDegreeMax) {
+        u64 total = 0;
+        CK(cudaMemcpyAsync(&total, h->in_off + n, sizeof(u64), cudaMemcpyDeviceToHost, h->stream));
+        CK(cudaStreamSynchronize(h->stream));
+        *counted = total == m;
+    }
+    if (m && *counted) {
+        k_scatter_in<<<h->grid, kThreads, 0, h->stream>>>(h->out_off, h->out_adj, n, h->wshift,
+                                                          h->in_off, cursor, h->in_adj);
+        CK(cudaGetLastError());
+    }
+    *sums = cnt;
+    return SSSP_OK;
+}
+
+// The device transposition with 64-bit counts and no classes.
+int transpose_plain(sssp_graph* h) {
+    const u32 n = h->n;
+    const u64 cntn = (u64)n + 1;
+    u64 *cnt = nullptr, *cursor = nullptr, *scan = nullptr;
+    Pool tmp;
+    tmp.al = h->gpool.al;
+    int rc = tmp.get(&cnt, cntn);
+    if (rc == SSSP_OK) rc = tmp.get(&cursor, cntn);
+    if (rc == SSSP_OK) rc = tmp.get(&scan, (cntn + kScanTile - 1) / kScanTile + 1);
+    if (rc == SSSP_OK) {
+        cudaError_t e = cudaMemsetAsync(cnt, 0, sizeof(u64) * cntn, h->stream);
+        if (e == cudaSuccess && h->m) {
+            k_count_in_plain<<<h->grid, kThreads, 0, h->stream>>>(h->out_adj, h->m, cnt);
+            e = cudaGetLastError();
+        }
+        if (e == cudaSuccess) rc = scan_excl(cnt, cntn, h->in_off, scan, h->stream);
+        if (rc == SSSP_OK && e == cudaSuccess)
+            e = cudaMemcpyAsync(cursor, h->in_off, sizeof(u64) * cntn, cudaMemcpyDeviceToDevice,
+                                h->stream);
+        if (rc == SSSP_OK && e == cudaSuccess && h->m) {
+            k_scatter_in_plain<<<h->grid, kThreads, 0, h->stream>>>(h->out_off, h->out_adj, n,
+                                                                    cursor, h->in_adj);
+            e = cudaGetLastError();
+        }
+        const cudaError_t es = cudaStreamSynchronize(h->stream);
+        if (rc == SSSP_OK && (e != cudaSuccess || es != cudaSuccess)) rc = SSSP_E_CUDA;
+        if (rc == SSSP_E_CUDA) (void)cudaGetLastError();
+    }
+    tmp.release();
+    return rc;
+}
+
 // Builds the graph on the device from arrays that sssp_create has checked
 // (wmax: their largest weight).
 int create_impl(sssp_graph* h, u32 n, u64 m, const u64* row_ptr, const u32* col, const u32* w,
@@ -693,38 +766,14 @@ int create_impl(sssp_graph* h, u32 n, u64 m, const u64* row_ptr, const u32* col,
                            cudaMemcpyHostToDevice, h->stream));
         RC(upload_adj(h, row, w_in, m, h->in_adj));
     } else {
-        // K0: transpose on the device (histogram, exclusive scan, scatter), the
-        // in-edges of a vertex in order of weight class.  (In-edges that the
-        // caller gives stay as they are.)
-        u64 *deg = nullptr, *sums = nullptr;
-        u32* cursor = nullptr;
-        const u64 cntn = (u64)n + 1, ncls = (u64)kClasses * n;
-        h->wshift = h->wmax >> 4 ? bits_for(h->wmax) - 4 : 0;
-        rc = tmp.get(&cnt, ncls);
-        if (rc == SSSP_OK) rc = tmp.get(&deg, cntn);
-        if (rc == SSSP_OK) rc = tmp.get(&cursor, ncls);
-        if (rc == SSSP_OK) rc = tmp.get(&sums, (cntn + kScanTile - 1) / kScanTile + 1);
-        cudaError_t e = cudaSuccess;
-        if (rc == SSSP_OK) {
-            e = cudaMemsetAsync(cnt, 0, sizeof(u32) * ncls, h->stream);
-            if (e == cudaSuccess) e = cudaMemsetAsync(deg + n, 0, sizeof(u64), h->stream);
-            if (e == cudaSuccess && m) {
-                k_count_in<<<h->grid, kThreads, 0, h->stream>>>(h->out_adj, m, h->wshift, cnt);
-                e = cudaGetLastError();
-            }
-            if (e == cudaSuccess) {
-                k_class_sums<<<h->grid, kThreads, 0, h->stream>>>(cnt, n, cursor, deg);
-                e = cudaGetLastError();
-            }
-            if (e == cudaSuccess) rc = scan_excl(deg, cntn, h->in_off, sums, h->stream);
-            if (rc == SSSP_OK && e == cudaSuccess && m) {
-                k_scatter_in<<<h->grid, kThreads, 0, h->stream>>>(h->out_off, h->out_adj, n,
-                                                                  h->wshift, h->in_off, cursor,
-                                                                  h->in_adj);
-                e = cudaGetLastError();
-            }
+        // K0: transpose on the device.  (In-edges that the caller gives stay as
+        // they are.)
+        bool counted = false;
+        rc = transpose_by_class(h, tmp, &cnt, &counted);
+        if (rc == SSSP_OK && !counted) {
+            cnt = nullptr;
+            rc = transpose_plain(h);
         }
-        if (rc == SSSP_OK && e != cudaSuccess) rc = SSSP_E_CUDA;
     }
     if (rc == SSSP_OK) rc = gp.get(&h->inw, n);
     if (rc == SSSP_OK) rc = gp.get(&h->vd, n);

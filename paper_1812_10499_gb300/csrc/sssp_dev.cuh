@@ -22,6 +22,13 @@ constexpr u64 kFixed = 1ull << 63;
 constexpr u64 kCMask = kFixed - 1;
 constexpr u32 kNoOutW = 0xFFFFFFFFu;   // vertex without out-edges
 
+// A degree as it is kept beside other words.  Parallel edges can give a vertex
+// kDegreeMax edges or more; such a degree is taken from the offsets.
+constexpr u32 kDegreeMax = 0xFFFFFFFFu;
+__host__ __device__ __forceinline__ u32 degree_word(u64 d) {
+    return d < kDegreeMax ? (u32)d : kDegreeMax;
+}
+
 // One vertex of one query.  cf[] is double-buffered by round parity: round r
 // reads cf[r & 1] (the lower bounds before the round: Jacobi update, SP_4
 // step 4 "in parallel") and writes cf[(r & 1) ^ 1].
@@ -29,7 +36,8 @@ struct __align__(32) VRec {
     u64 dp;        // packed upper bound D (atomicMin target)
     u64 cf[2];     // lower bound C | kFixed
     u32 outw;      // outWeight (Fig. SP_3 / SP_4 declarations), kNoOutW if none
-    u32 indeg;     // in-degree (decides the work list of a newly discovered vertex)
+    u32 indeg;     // in-degree (decides the work list of a newly discovered vertex),
+                   // as degree_word
 };
 static_assert(sizeof(VRec) == 32, "VRec must be one 32-byte sector");
 
@@ -66,12 +74,41 @@ __host__ __device__ __forceinline__ u32 wclass(u32 w, u32 shift) {
 // in an array of their own, a sector more, had cost as much as they saved.
 struct __align__(32) VDesc {
     u64 ib;                 // first in-edge
-    u32 deg, odeg;          // in-degree, out-degree
+    u32 deg, odeg;          // in-degree, out-degree (degree_word)
     u32 outw, inw;          // least out- and in-weight (kNoOutW: none)
     u32 cum[2];             // byte k: the in-edges in weight classes 0 to k; above 255
                             // in-edges, in 255ths of them, rounded up
 };
 static_assert(sizeof(VDesc) == 32, "VDesc must be one 32-byte sector");
+
+// The description of a vertex from its first in-edge, degrees and least weights;
+// sums: its in-edges in weight classes 0 to k (kClasses words), or nullptr when
+// the row is in no such order (every prefix is the whole row then, as it is for
+// a degree that its word does not hold).
+__host__ __device__ __forceinline__ VDesc make_vdesc(u64 ib, u64 deg, u64 odeg, u32 outw, u32 inw,
+                                                     const u32* sums) {
+    VDesc d;
+    d.ib = ib;
+    d.deg = degree_word(deg);
+    d.odeg = degree_word(odeg);
+    d.outw = outw;
+    d.inw = inw;
+    d.cum[0] = d.cum[1] = 0;
+    for (u32 k = 0; k < kClasses; ++k) {
+        const u32 c = sums && d.deg != kDegreeMax ? sums[k] : d.deg;
+        const u32 b = d.deg <= 255 ? c : (u32)(((u64)c * 255 + d.deg - 1) / d.deg);
+        d.cum[k >> 2] |= b << (8 * (k & 3));
+    }
+    return d;
+}
+
+// At least the in-edges with weights up to wtop, from the start of the row.
+__host__ __device__ __forceinline__ u32 light_prefix(const VDesc& x, u32 wtop, u32 shift) {
+    const u32 k = wclass(wtop, shift);
+    const u32 b = ((k & 4 ? x.cum[1] : x.cum[0]) >> (8 * (k & 3))) & 255u;
+    if (x.deg <= 255) return b < x.deg ? b : x.deg;
+    return (u32)(((u64)b * x.deg + 254) / 255);
+}
 
 // Read-only description of one query's graph.
 struct InstDesc {

@@ -53,6 +53,9 @@ __global__ void k_finalize_multi(RoundParams P, u64 nrec, u64* dist);
 __global__ void k_interleave(const u32* col, const u32* w, u64 m, uint2* adj);
 __global__ void k_find_loop(const u64* out_off, const uint2* out_adj, u32 n, u32* flag);
 __global__ void k_count_in(const uint2* adj, u64 m, u32 wshift, u32* cnt);
+__global__ void k_count_in_plain(const uint2* adj, u64 m, u64* cnt);
+__global__ void k_scatter_in_plain(const u64* out_off, const uint2* out_adj, u32 n, u64* cursor,
+                                   uint2* in_adj);
 __global__ void k_class_sums(u32* cnt, u32 n, u32* cursor, u64* deg);
 __global__ void k_vdesc(const u64* out_off, const u64* in_off, const u32* outw, const u32* inw,
                         const u32* sums, u32 n, VDesc* vd);

@@ -285,6 +285,11 @@ __device__ __forceinline__ void put_hub(const RoundParams& P, u64* pk, uint2* li
     for (u32 k = first; k < end; ++k) cmap[k] = idx;
 }
 
+// The out-degree of vertex v, whose description holds it as `word`.
+__device__ __forceinline__ u64 out_degree(const InstDesc& d, u32 v, u32 word) {
+    return word == kDegreeMax ? d.out_off[v + 1] - d.out_off[v] : word;
+}
+
 // Entry of hub list `list` (n entries) that chunk c belongs to: from the
 // chunk map, else by binary search over the entries' first chunks.
 __device__ __forceinline__ u32 hub_entry(const RoundParams& P, const uint2* list, const u32* cmap,
@@ -717,19 +722,13 @@ __device__ __forceinline__ VDesc vertex_desc(const RoundParams& P, const InstDes
         x.cum[1] = b.w;
     } else {
         x.ib = d.in_off[v];
-        x.deg = (u32)(d.in_off[v + 1] - x.ib);
-        x.odeg = (u32)(d.out_off[v + 1] - d.out_off[v]);
+        x.deg = degree_word(d.in_off[v + 1] - x.ib);
+        x.odeg = degree_word(d.out_off[v + 1] - d.out_off[v]);
         x.outw = outw_of<L>(d, r, v);
         x.inw = P.cheap ? d.inw[v] : 0u;
         x.cum[0] = x.cum[1] = kFull;
     }
     return x;
-}
-// At least the in-edges with weights up to wtop, from the start of the row.
-__device__ __forceinline__ u32 light_prefix(const VDesc& x, u32 wtop, u32 shift) {
-    const u32 k = wclass(wtop, shift);
-    const u32 b = ((k & 4 ? x.cum[1] : x.cum[0]) >> (8 * (k & 3))) & 255u;
-    return x.deg <= 255 ? min(b, x.deg) : (u32)(((u64)b * x.deg + 254) / 255);
 }
 
 // Starts gathering the source states of the nb in-edges in adjacency slot as
@@ -909,6 +908,10 @@ __device__ __forceinline__ void relax_consume(const RoundParams& P, InstCache<ty
                 deg = d.in_off[pd.yl[i] + 1] - d.in_off[pd.yl[i]];
             } else {
                 deg = pd.deg[i];
+                if (deg == kDegreeMax) {
+                    const InstDesc& d = MULTI ? P.idesc[pd.inst[i]] : P.g;
+                    deg = d.in_off[pd.yl[i] + 1] - d.in_off[pd.yl[i]];
+                }
             }
             put_hub(P, &P.ctl->AHpk[cur], P.L.AH[cur], P.L.AC[cur], pd.gy[i], deg);
         }
@@ -1272,7 +1275,9 @@ __device__ void cup_small(const RoundParams& P, InstCache<typename L::Term>* ic,
     const bool fs = fx && x.odeg <= P.hub;
     if (P.lc) wq_push(P, qf, &P.ctl->nFX[nxt], P.L.FX[nxt], valid && fix, g, lane);
     else wq_push(P, qf, &P.ctl->nFS[nxt], P.L.FS[nxt], fs, g, lane);
-    if (fx && !fs) put_hub(P, &P.ctl->FHpk[nxt], P.L.FH[nxt], P.L.FC[nxt], g, x.odeg);
+    if (fx && !fs)
+        put_hub(P, &P.ctl->FHpk[nxt], P.L.FH[nxt], P.L.FC[nxt], g,
+                out_degree(MULTI ? P.idesc[inst] : P.g, yloc, x.odeg));
     wq_push(P, qa, &P.ctl->nAS[nxt], P.L.AS[nxt], sv, g, lane);
     const u64 tsum = x.outw == kNoOutW ? P.dinf : dy + x.outw;
     if (MULTI) {
@@ -1302,8 +1307,9 @@ __device__ void cup_hub(const RoundParams& P, InstCache<typename L::Term>* ic, W
     }
     const u32 yloc = g - (u32)d.base;
     const VDesc x = vertex_desc<L>(P, d, yloc, L::rec(P) + g);
-    const u64 ib = x.ib, ie = ib + x.deg;
-    const u32 nch = (u32)(((u64)x.deg + P.chunk - 1) / P.chunk);   // as counted by put_hub
+    const bool whole = x.deg == kDegreeMax;    // its degree is in the offsets
+    const u64 ib = x.ib, ie = whole ? d.in_off[yloc + 1] : ib + x.deg;
+    const u32 nch = (u32)((ie - ib + P.chunk - 1) / P.chunk);   // as counted by put_hub
     const u64 cb = ib + (u64)k * P.chunk + ((P.chunk * part) >> ps);
     const u64 ce = umin64(ib + (u64)k * P.chunk + ((P.chunk * (part + 1)) >> ps), ie);
     const typename L::Bounds bd = L::bounds(thr, minD);
@@ -1313,14 +1319,14 @@ __device__ void cup_hub(const RoundParams& P, InstCache<typename L::Term>* ic, W
     bool fix_now = false;
     const u64 dh = L::ld_dc(L::rec(P) + g, cur).x >> P.vbits;
     if (P.cheap) fix_now = cheap_rules_fix(dh, x.inw, thr, minD);
-    if (L::kPred && !fix_now) fix_now = P.pcnt[g] == 0u;
+    if (L::kPred && !fix_now) fix_now = !whole && P.pcnt[g] == 0u;
     u32 n = (ce > cb && !fix_now) ? (u32)(ce - cb) : 0u;
     if (lane == 0) a.edges += n;
     const u64 lim = weight_limit(dh, minD);
     const u32 wtop = (u32)umin64(lim - 1, kFull);
     if (lim == 0) {
         n = 0;
-    } else if (n) {
+    } else if (n && !whole) {
         const u64 end = ib + light_prefix(x, wtop, d.wshift);
         n = end > cb ? (u32)umin64(n, end - cb) : 0u;
     }
@@ -1385,7 +1391,8 @@ __device__ void cup_hub(const RoundParams& P, InstCache<typename L::Term>* ic, W
     }
     if (front) {
         if (x.odeg <= P.hub) put_small(P, P.L.FS[nxt], atomicAdd(&P.ctl->nFS[nxt], 1u), g);
-        else put_hub(P, &P.ctl->FHpk[nxt], P.L.FH[nxt], P.L.FC[nxt], g, x.odeg);
+        else
+            put_hub(P, &P.ctl->FHpk[nxt], P.L.FH[nxt], P.L.FC[nxt], g, out_degree(d, yloc, x.odeg));
         if (MULTI) inst_count(P, ic, inst, nxt);
         else an.nfix++;
     }

@@ -35,7 +35,7 @@ __global__ void k_init_records(VRec* rec, VRecN* recn, int* fround, const u32* o
             r.cf[0] = 0;
             r.cf[1] = 0;
             r.outw = outw[v];
-            r.indeg = (u32)(in_off[v + 1] - in_off[v]);
+            r.indeg = degree_word(in_off[v + 1] - in_off[v]);
             rec[v] = r;
         }
         fround[v] = -1;
@@ -68,7 +68,7 @@ __global__ void k_init_records_multi(RoundParams P, u64 nrec, u32 first_page, u3
             r.cf[0] = 0;
             r.cf[1] = 0;
             r.outw = d.outw[v];
-            r.indeg = (u32)(d.in_off[v + 1] - d.in_off[v]);
+            r.indeg = degree_word(d.in_off[v + 1] - d.in_off[v]);
             P.rec[g] = r;
         }
         P.fround[g] = -1;
@@ -159,6 +159,24 @@ __global__ void k_count_in(const uint2* adj, u64 m, u32 wshift, u32* cnt) {
     }
 }
 
+// The plain transposition's counts, in 64 bits and without classes, and its scatter
+// (one warp per source vertex).
+__global__ void k_count_in_plain(const uint2* adj, u64 m, u64* cnt) {
+    for (u64 i = blockIdx.x * (u64)blockDim.x + threadIdx.x; i < m;
+         i += (u64)gridDim.x * blockDim.x)
+        atomicAdd(&cnt[adj[i].x], 1ull);
+}
+__global__ void k_scatter_in_plain(const u64* out_off, const uint2* out_adj, u32 n, u64* cursor,
+                                   uint2* in_adj) {
+    const u32 lane = threadIdx.x & 31u;
+    for (u64 u = (blockIdx.x * (u64)blockDim.x + threadIdx.x) >> 5; u < n;
+         u += ((u64)gridDim.x * blockDim.x) >> 5)
+        for (u64 k = out_off[u] + lane; k < out_off[u + 1]; k += 32) {
+            const uint2 e = out_adj[k];
+            in_adj[atomicAdd(&cursor[e.x], 1ull)] = make_uint2((u32)u, e.y);
+        }
+}
+
 // The class counts of every vertex: to sums up to and with each class (in
 // place), to sums before it (cursor), and their total (deg).
 __global__ void k_class_sums(u32* cnt, u32 n, u32* cursor, u64* deg) {
@@ -188,21 +206,9 @@ __global__ void k_class_sums(u32* cnt, u32 n, u32* cursor, u64* deg) {
 __global__ void k_vdesc(const u64* out_off, const u64* in_off, const u32* outw, const u32* inw,
                         const u32* sums, u32 n, VDesc* vd) {
     for (u64 v = blockIdx.x * (u64)blockDim.x + threadIdx.x; v < n;
-         v += (u64)gridDim.x * blockDim.x) {
-        VDesc d;
-        d.ib = in_off[v];
-        d.deg = (u32)(in_off[v + 1] - d.ib);
-        d.odeg = (u32)(out_off[v + 1] - out_off[v]);
-        d.outw = outw[v];
-        d.inw = inw[v];
-        d.cum[0] = d.cum[1] = 0;
-        for (u32 k = 0; k < kClasses; ++k) {
-            const u32 c = sums ? sums[kClasses * v + k] : d.deg;
-            const u32 b = d.deg <= 255 ? c : (u32)(((u64)c * 255 + d.deg - 1) / d.deg);
-            d.cum[k >> 2] |= b << (8 * (k & 3));
-        }
-        vd[v] = d;
-    }
+         v += (u64)gridDim.x * blockDim.x)
+        vd[v] = make_vdesc(in_off[v], in_off[v + 1] - in_off[v], out_off[v + 1] - out_off[v],
+                           outw[v], inw[v], sums ? sums + kClasses * v : nullptr);
 }
 
 // One warp per source vertex scatters its out-edges into the in-lists, each into
