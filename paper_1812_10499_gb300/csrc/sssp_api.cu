@@ -476,6 +476,7 @@ int init_single_context(sssp_graph* h) {
     c.tail_ctas = h->tail_ctas;
     RoundParams& P = c.P;
     P.tail_items = h->tail_items;
+    P.tail_chunks = small_chunks(h->opt.hub_degree);
     P.small = h->n <= 0x7FFFFFFFu && h->m <= 0xFFFFFFFFull;
     P.g.out_off = h->out_off;
     P.g.out_adj = h->out_adj;

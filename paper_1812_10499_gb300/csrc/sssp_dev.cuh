@@ -223,6 +223,7 @@ struct RoundParams {
     u32 trace_cap;              // entries of `trace`
     u32 trace_base;             // round number of the first traced round
     u32 tail_items;             // cluster tail kernel: most work items a round may have
+    u32 tail_chunks;            // small-round kernel: most hub chunks a list may have
     u32 small;                  // 1: single query whose ids fit 31 bits and edges 32 bits
                                 // (the small-round kernel's list entries)
     u32 lc;                     // 1: label-correcting relaxation (SP_4 step 3 as printed):

@@ -27,6 +27,12 @@ struct TailKernel {
     size_t smem;
 };
 TailKernel small_kernel(bool narrow, bool win);
+// Most hub chunks in a round of k_small: 16, or, with a hub degree below 256, as many as
+// hold 4096 edges if every one is a vertex just above it; such hubs are short rows to
+// k_small, which 16 of them do not fill.  (Hub degree 4, 16 chunks -> this rule: random
+// n = 300 260 -> 127 us, n = 4096 602 -> 412 us, R-MAT 15 593 -> 497 us; degree 16, random
+// n = 20000 747 -> 540 us; half of it, 2048 edges, 602 us there.)
+inline u32 small_chunks(u32 hub_degree) { return std::max(16u, 4096u / hub_degree); }
 TailKernel tail_kernel(bool multi, bool narrow, const RoundParams& P);
 const void* barrier_selftest_fn();
 u32 tail_cluster_ctas();

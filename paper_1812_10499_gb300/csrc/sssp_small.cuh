@@ -37,7 +37,6 @@ constexpr u32 kSmallCTAs = kTailCTAs;
 constexpr u32 kSmallThreads = 512;
 constexpr u32 kSmallWarps = kSmallThreads / 32;
 constexpr u32 kSmallCap = 1024;      // entries of a CTA's active list, and of its frontier
-constexpr u32 kSmallChunks = 16;     // most 1024-edge chunks of hub vertices per list
 // Edges in flight per lane.  1: random n = 4096 and R-MAT tails 7-17% slower
 // (degrees above the group's lanes); 4: grids 7% slower (empty slots).
 constexpr u32 kSmallU = 2;
@@ -645,11 +644,11 @@ __device__ __forceinline__ void small_phase_bounds(const RoundParams& P, SmallSh
 // Whether round ctl->round starts in this kernel: the loop is running and not
 // past its stop round, the frontier and the active set each make at most
 // P.tail_items work items (32-entry tiles plus hub chunks) and fit the lists,
-// and few of them are hub chunks.  Every CTA takes the same decision.
+// and few of them are hub chunks (P.tail_chunks).  Every CTA takes the same decision.
 __device__ __forceinline__ bool small_fits(const RoundParams& P, u32 items, u32 entries,
                                            u32 chunks) {
     return items <= P.tail_items && entries <= kSmallCTAs * (kSmallCap * 3 / 4) &&
-           chunks <= kSmallChunks;
+           chunks <= P.tail_chunks;
 }
 
 template <class S, bool WIN>
