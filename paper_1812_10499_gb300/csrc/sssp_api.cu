@@ -579,6 +579,20 @@ void strip_loops(u32 n, const u64* off, const u32* idx, const u32* w, std::vecto
     o2[n] = i2.size();
 }
 
+// Whether a CSR holds a self-loop.
+bool has_loop(u32 n, const u64* off, const u32* idx) {
+    for (u32 u = 0; u < n; ++u)
+        for (u64 k = off[u]; k < off[u + 1]; ++k)
+            if (idx[k] == u) return true;
+    return false;
+}
+
+// Graphs of up to this many edges are looked over for self-loops on the host, before
+// the upload: the device's answer costs about 25 us whatever the size (allocation,
+// kernel, wait), and loops found by it a second upload.  Creating random n = 300 with
+// self-loops 796 -> 703 us.
+constexpr u64 kHostLoopEdges = 1u << 15;
+
 // Whether the uploaded out-edges hold a self-loop (waits for the stream).
 int has_loop(sssp_graph* h, u32 n, bool* found) {
     Pool tmp;
@@ -634,14 +648,15 @@ int upload_adj(sssp_graph* h, const u32* idx, const u32* w, u64 m, uint2* adj) {
 int transpose_by_class(sssp_graph* h, Pool& tmp, u32** sums, bool* counted) {
     const u32 n = h->n;
     const u64 m = h->m, cntn = (u64)n + 1, ncls = (u64)kClasses * n;
+    const u64 sums_n = (cntn + kScanTile - 1) / kScanTile + 1;
     u32 *cnt = nullptr, *cursor = nullptr;
-    u64 *deg = nullptr, *scan = nullptr;
+    u64* deg = nullptr;
     *counted = true;
     h->wshift = h->wmax >> 4 ? bits_for(h->wmax) - 4 : 0;
     RC(tmp.get(&cnt, ncls));
-    RC(tmp.get(&deg, cntn));
     RC(tmp.get(&cursor, ncls));
-    RC(tmp.get(&scan, (cntn + kScanTile - 1) / kScanTile + 1));
+    RC(tmp.get(&deg, cntn + sums_n));
+    u64* scan = deg + cntn;
     CK(cudaMemsetAsync(cnt, 0, sizeof(u32) * ncls, h->stream));
     CK(cudaMemsetAsync(deg + n, 0, sizeof(u64), h->stream));
     if (m) {
@@ -718,6 +733,27 @@ int create_impl(sssp_graph* h, u32 n, u64 m, const u64* row_ptr, const u32* col,
         h->dinf = (~0ull) >> 32;
     }
 
+    // Self-loops (rare) are dropped on the host.
+    std::vector<u64> o2, c2;
+    std::vector<u32> i2, w2, r2, wi2;
+    auto drop_loops = [&]() -> int {
+        strip_loops(n, row_ptr, col, w, o2, i2, w2);
+        row_ptr = o2.data();
+        col = i2.data();
+        w = w2.data();
+        m = o2[n];
+        if (csc_given) {
+            strip_loops(n, col_ptr, row, w_in, c2, r2, wi2);
+            col_ptr = c2.data();
+            row = r2.data();
+            w_in = wi2.data();
+            if (c2[n] != m) return SSSP_E_INVAL;
+        }
+        return SSSP_OK;
+    };
+    const bool host_look = m <= kHostLoopEdges;
+    if (host_look && has_loop(n, row_ptr, col)) RC(drop_loops());
+
     CK(cudaStreamCreateWithFlags(&h->stream, cudaStreamNonBlocking));
     h->grid = occupancy_grid(h->device, h->opt);
     h->grid_cup = occupancy_grid(h->device, h->opt, true);
@@ -736,24 +772,15 @@ int create_impl(sssp_graph* h, u32 n, u64 m, const u64* row_ptr, const u32* col,
     CK(cudaMemcpyAsync(h->out_off, row_ptr, sizeof(u64) * ((size_t)n + 1), cudaMemcpyHostToDevice,
                        h->stream));
     RC(upload_adj(h, col, w, m, h->out_adj));
-    // Self-loops (rare) are dropped on the host and the edges uploaded again.
-    std::vector<u64> o2, c2;
-    std::vector<u32> i2, w2, r2, wi2;
-    bool loops = false;
-    RC(has_loop(h, n, &loops));
-    if (loops) {
-        strip_loops(n, row_ptr, col, w, o2, i2, w2);
-        m = o2[n];
-        if (csc_given) {
-            strip_loops(n, col_ptr, row, w_in, c2, r2, wi2);
-            col_ptr = c2.data();
-            row = r2.data();
-            w_in = wi2.data();
-            if (c2[n] != m) return SSSP_E_INVAL;
+    if (!host_look) {
+        bool loops = false;
+        RC(has_loop(h, n, &loops));
+        if (loops) {
+            RC(drop_loops());
+            CK(cudaMemcpyAsync(h->out_off, row_ptr, sizeof(u64) * ((size_t)n + 1),
+                               cudaMemcpyHostToDevice, h->stream));
+            RC(upload_adj(h, col, w, m, h->out_adj));
         }
-        CK(cudaMemcpyAsync(h->out_off, o2.data(), sizeof(u64) * ((size_t)n + 1),
-                           cudaMemcpyHostToDevice, h->stream));
-        RC(upload_adj(h, i2.data(), w2.data(), m, h->out_adj));
     }
     h->n = n;
     h->m = m;
@@ -776,9 +803,11 @@ int create_impl(sssp_graph* h, u32 n, u64 m, const u64* row_ptr, const u32* col,
             rc = transpose_plain(h);
         }
     }
-    if (rc == SSSP_OK) rc = gp.get(&h->inw, n);
-    if (rc == SSSP_OK) rc = gp.get(&h->vd, n);
+    unsigned char* desc = nullptr;   // the vertices' descriptions, then their inWeights
+    if (rc == SSSP_OK) rc = gp.get(&desc, (size_t)n * (sizeof(VDesc) + sizeof(u32)));
     if (rc == SSSP_OK) {
+        h->vd = reinterpret_cast<VDesc*>(desc);
+        h->inw = reinterpret_cast<u32*>(desc + (size_t)n * sizeof(VDesc));
         k_outw<<<h->grid, kThreads, 0, h->stream>>>(h->out_off, h->out_adj, n, h->outw);
         // inWeight: the same reduction over the in-edges
         k_outw<<<h->grid, kThreads, 0, h->stream>>>(h->in_off, h->in_adj, n, h->inw);
@@ -792,9 +821,10 @@ int create_impl(sssp_graph* h, u32 n, u64 m, const u64* row_ptr, const u32* col,
     RC(rc);
     // The graph's degree statistics (its class in the tuning cache), then
     // the state that depends on the tuning.
-    RC(count_hubs(h, h->opt.hub_degree, &h->hubs_out, &h->hubs_in, &h->max_out, &h->max_in));
+    const u32 hub = h->opt.hub_degree;
+    RC(count_hubs(h, hub, &h->hubs_out, &h->hubs_in, &h->max_out, &h->max_in));
     resolve_tuning(h);
-    RC(apply_tuning(h));
+    RC(apply_tuning(h, h->opt.hub_degree == hub));
     return SSSP_OK;
 }
 
@@ -824,8 +854,9 @@ int count_hubs(sssp_graph* h, u32 hub, u32* hubs_out, u32* hubs_in, u32* max_out
 
 // State that depends on the tuning (hub degree, chunk size, CTAs per SM,
 // cluster-tail thresholds): the round kernels' grids, the compact layout's
-// in-hub flags, the hub counts, and the solve contexts (rebuilt).
-int apply_tuning(sssp_graph* h) {
+// in-hub flags, the hub counts (unless they are of this hub degree: counted), and
+// the solve contexts (rebuilt).
+int apply_tuning(sssp_graph* h, bool counted) {
     const u32 n = h->n;
     CK(cudaStreamSynchronize(h->stream));
     h->grid = occupancy_grid(h->device, h->opt);
@@ -837,7 +868,8 @@ int apply_tuning(sssp_graph* h) {
                                                          h->outw_pack);
         CK(cudaGetLastError());
     }
-    RC(count_hubs(h, h->opt.hub_degree, &h->hubs_out, &h->hubs_in, nullptr, nullptr));
+    if (!counted)
+        RC(count_hubs(h, h->opt.hub_degree, &h->hubs_out, &h->hubs_in, nullptr, nullptr));
     h->single.destroy();
     h->single = Context();
     if (h->batch) {

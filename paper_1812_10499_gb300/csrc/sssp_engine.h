@@ -269,7 +269,7 @@ struct sssp_graph {
 namespace sssp {
 namespace engine {
 int count_hubs(sssp_graph* h, u32 hub, u32* hubs_out, u32* hubs_in, u32* max_out, u32* max_in);
-int apply_tuning(sssp_graph* h);
+int apply_tuning(sssp_graph* h, bool counted = false);
 void resolve_tuning(sssp_graph* h);
 int enqueue_single(sssp_graph* h, u32 source, u32 max_rounds, cudaStream_t st, u64* dist_dev,
                    u32* parent_dev, int* fround_dev, u64* lower_dev, u32 target);

@@ -78,7 +78,8 @@ cudaError_t set_tail_attributes(const TailKernel& k) {
 }
 
 // Raises the dynamic shared-memory limit of the round kernels of one family
-// (default or counting) and allows the tail kernels' 16-CTA cluster.
+// (default or counting) and allows k_tail's 16-CTA cluster (k_small's are set up
+// in tail_cluster_ctas alone: this function runs six times while a graph is created).
 cudaError_t set_attributes(bool pred) {
     cudaError_t e = cudaSuccess;
     for (int v = 0; v < 4 && e == cudaSuccess; ++v) {
@@ -95,7 +96,6 @@ cudaError_t set_attributes(bool pred) {
                                      cudaFuncAttributeMaxDynamicSharedMemorySize,
                                      (int)solve_smem_bytes(narrow));
         if (e == cudaSuccess) e = set_tail_attributes(list_tail(multi, narrow, pred));
-        if (e == cudaSuccess && !pred) e = set_tail_attributes(small_kernel(narrow, multi));
     }
     return e;
 }
@@ -166,10 +166,13 @@ cudaError_t pred_kernels_init() {
 // scheduled on the current device (the device loop then runs without it).
 u32 tail_cluster_ctas() {
     if (round_kernels_init() != cudaSuccess) return 0;
-    for (int v = 0; v < 4; ++v)
-        if (clusters_per_gpu(list_tail(v & 1, (v >> 1) & 1, false)) < 1 ||
-            clusters_per_gpu(small_kernel(v & 1, (v >> 1) & 1)) < 1)
+    for (int v = 0; v < 4; ++v) {
+        const TailKernel small = small_kernel(v & 1, (v >> 1) & 1);
+        if (set_tail_attributes(small) != cudaSuccess ||
+            clusters_per_gpu(list_tail(v & 1, (v >> 1) & 1, false)) < 1 ||
+            clusters_per_gpu(small) < 1)
             return 0;
+    }
     return kTailCTAs;
 }
 

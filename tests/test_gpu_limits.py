@@ -35,3 +35,41 @@ def test_small_hubs_stay_in_the_cluster_kernel(sssp_lib, layout, mode, delta, hu
     assert 0 < prof["tail_rounds"] <= rounds - 1
     if n == 250:
         assert prof["tail_rounds"] == rounds - 1
+
+
+class Budget:
+    """Device allocator hooks that count, and refuse what would pass a number of bytes."""
+
+    def __init__(self, P, nbytes=1 << 40):
+        import torch
+        self.live, self.left, self.calls = {}, nbytes, 0
+
+        def alloc(size, _ctx):
+            self.calls += 1
+            if size > self.left:
+                return None
+            t = torch.empty(max(size, 1), dtype=torch.uint8, device="cuda")
+            self.live[t.data_ptr()] = (t, size)
+            self.left -= size
+            return t.data_ptr()
+
+        def free(p, _ctx):
+            torch.cuda.synchronize()
+            self.left += self.live.pop(p)[1]
+
+        self.options = P.sssp_options_default()
+        self.options.alloc, self.options.free = P.ALLOC_FN(alloc), P.FREE_FN(free)
+
+
+@pytest.mark.parametrize("n", [2, 300, 4000])
+def test_allocations_of_a_small_graph(sssp_lib, n):
+    """Creating a small graph takes 31 allocations: 7 for the graph (five arrays, the
+    descriptions, the packed outWeights), 6 of scratch (two for the upload, three for the
+    transposition, the hub counts), 18 for the solve state; none to look for self-loops."""
+    P = sssp_lib
+    g = gg.random_graph(n, min(n - 1, 6), 1, 50, 2)
+    b = Budget(P)
+    h = P.sssp_create(g.n, g.row_ptr, g.col, g.w, options=b.options)
+    calls = b.calls
+    P.sssp_destroy(h)
+    assert calls <= 31 and not b.live
