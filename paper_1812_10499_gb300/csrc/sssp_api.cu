@@ -715,9 +715,12 @@ int transpose_plain(sssp_graph* h) {
 }
 
 // Builds the graph on the device from arrays that sssp_create has checked
-// (wmax: their largest weight).
+// (wmax: their largest weight).  lean: with as little device memory as the solves can
+// do with -- no vertex descriptions (32 bytes per vertex), so no weight classes (whose
+// counts take 64 bytes per vertex of scratch, where the plain ones take 16), and no
+// room for self-loops.
 int create_impl(sssp_graph* h, u32 n, u64 m, const u64* row_ptr, const u32* col, const u32* w,
-                const u64* col_ptr, const u32* row, const u32* w_in, u32 wmax) {
+                const u64* col_ptr, const u32* row, const u32* w_in, u32 wmax, bool lean) {
     const bool csc_given = col_ptr || row || w_in;
     h->vbits = std::max<u32>(1, bits_for((u64)n - 1));
     h->dinf = (~0ull) >> h->vbits;
@@ -751,7 +754,7 @@ int create_impl(sssp_graph* h, u32 n, u64 m, const u64* row_ptr, const u32* col,
         }
         return SSSP_OK;
     };
-    const bool host_look = m <= kHostLoopEdges;
+    const bool host_look = lean || m <= kHostLoopEdges;
     if (host_look && has_loop(n, row_ptr, col)) RC(drop_loops());
 
     CK(cudaStreamCreateWithFlags(&h->stream, cudaStreamNonBlocking));
@@ -797,22 +800,24 @@ int create_impl(sssp_graph* h, u32 n, u64 m, const u64* row_ptr, const u32* col,
         // K0: transpose on the device.  (In-edges that the caller gives stay as
         // they are.)
         bool counted = false;
-        rc = transpose_by_class(h, tmp, &cnt, &counted);
+        if (!lean) rc = transpose_by_class(h, tmp, &cnt, &counted);
         if (rc == SSSP_OK && !counted) {
             cnt = nullptr;
             rc = transpose_plain(h);
         }
     }
     unsigned char* desc = nullptr;   // the vertices' descriptions, then their inWeights
-    if (rc == SSSP_OK) rc = gp.get(&desc, (size_t)n * (sizeof(VDesc) + sizeof(u32)));
+    const size_t vd_bytes = lean ? 0 : (size_t)n * sizeof(VDesc);
+    if (rc == SSSP_OK) rc = gp.get(&desc, vd_bytes + (size_t)n * sizeof(u32));
     if (rc == SSSP_OK) {
-        h->vd = reinterpret_cast<VDesc*>(desc);
-        h->inw = reinterpret_cast<u32*>(desc + (size_t)n * sizeof(VDesc));
+        if (!lean) h->vd = reinterpret_cast<VDesc*>(desc);
+        h->inw = reinterpret_cast<u32*>(desc + vd_bytes);
         k_outw<<<h->grid, kThreads, 0, h->stream>>>(h->out_off, h->out_adj, n, h->outw);
         // inWeight: the same reduction over the in-edges
         k_outw<<<h->grid, kThreads, 0, h->stream>>>(h->in_off, h->in_adj, n, h->inw);
-        k_vdesc<<<h->grid, kThreads, 0, h->stream>>>(h->out_off, h->in_off, h->outw, h->inw, cnt, n,
-                                                     h->vd);
+        if (!lean)
+            k_vdesc<<<h->grid, kThreads, 0, h->stream>>>(h->out_off, h->in_off, h->outw, h->inw,
+                                                         cnt, n, h->vd);
         if (cudaGetLastError() != cudaSuccess) rc = SSSP_E_CUDA;
     }
     if (cudaStreamSynchronize(h->stream) != cudaSuccess && rc == SSSP_OK) rc = SSSP_E_CUDA;
@@ -1205,23 +1210,27 @@ int sssp_create(uint32_t n, uint64_t m, const uint64_t* row_ptr, const uint32_t*
         (void)cudaGetLastError();
         return SSSP_E_CUDA;
     }
-    sssp_graph* h = new (std::nothrow) sssp_graph();
-    if (!h) return SSSP_E_NOMEM;
-    h->device = dev;
-    h->opt = o;
-    h->opt.device = dev;
-    h->tune_auto = tune_auto;
-    h->gpool.al = Allocator{o.alloc, o.free, o.alloc_ctx};
-    int rc;
-    {
-        DeviceGuard dg(dev);
-        rc = create_impl(h, n, m, reinterpret_cast<const u64*>(row_ptr), col, w,
-                         reinterpret_cast<const u64*>(col_ptr), row, w_in, wmax);
-        if (rc != SSSP_OK) destroy_impl(h);
-    }
-    if (rc != SSSP_OK) {
+    // With everything that speeds the solves up; where device memory does not hold that,
+    // once more without.
+    sssp_graph* h = nullptr;
+    for (const bool lean : {false, true}) {
+        h = new (std::nothrow) sssp_graph();
+        if (!h) return SSSP_E_NOMEM;
+        h->device = dev;
+        h->opt = o;
+        h->opt.device = dev;
+        h->tune_auto = tune_auto;
+        h->gpool.al = Allocator{o.alloc, o.free, o.alloc_ctx};
+        int rc;
+        {
+            DeviceGuard dg(dev);
+            rc = create_impl(h, n, m, reinterpret_cast<const u64*>(row_ptr), col, w,
+                             reinterpret_cast<const u64*>(col_ptr), row, w_in, wmax, lean);
+            if (rc != SSSP_OK) destroy_impl(h);
+        }
+        if (rc == SSSP_OK) break;
         delete h;
-        return rc;
+        if (lean || rc != SSSP_E_NOMEM) return rc;
     }
     *out = h;
     return SSSP_OK;

@@ -73,3 +73,42 @@ def test_allocations_of_a_small_graph(sssp_lib, n):
     calls = b.calls
     P.sssp_destroy(h)
     assert calls <= 31 and not b.live
+
+
+@pytest.mark.parametrize("given_csc", [False, True])
+@pytest.mark.parametrize("loops", [False, True])
+def test_graph_that_fits_without_descriptions(sssp_lib, loops, given_csc):
+    """A memory budget that holds the graph (28 bytes per vertex and 16 per edge), its
+    compact state (52 per vertex), the lower bounds on their way to the host (8 per vertex)
+    and the control slots, but no vertex descriptions: the graph is created, self-loops
+    take no room, and every output is the oracle's.  A budget that does not hold the
+    graph gives SSSP_E_NOMEM and everything is handed back."""
+    P = sssp_lib
+    g = gg.grid(300, 200, 1, 900, 5)
+    full = g
+    if loops:
+        src, col, w = g.edges()
+        every = np.arange(g.n, dtype=np.uint32)
+        full = gg.from_edges(g.n, np.stack([np.concatenate([src, every]), np.concatenate([col, every]),
+                                            np.concatenate([w, np.ones_like(every)])], 1).tolist())
+    csc = {}
+    if given_csc:
+        s, c, ww = full.edges()
+        order = np.argsort(c, kind="stable")
+        ptr = np.concatenate([[0], np.cumsum(np.bincount(c, minlength=g.n))])
+        csc = dict(col_ptr=ptr.astype(np.uint64), row=s[order], w_in=ww[order])
+    b = Budget(P, 89 * g.n + 16 * g.m + (1 << 17))
+    h = P.sssp_create(g.n, full.row_ptr, full.col, full.w, options=b.options, **csc)
+    try:
+        assert P.sssp_num_edges(h) == g.m
+        out = P.sssp_solve_ex(h, 123, parent=True, fixed_round=True, lower=True)
+    finally:
+        P.sssp_destroy(h)
+    assert not b.live
+    ref = oracle.round_r(g, 123)
+    assert np.array_equal(out["dist"], ref.dist) and np.array_equal(out["parent"], ref.parent)
+    assert np.array_equal(out["fixed_round"], ref.fixed_round) and np.array_equal(out["lower"], ref.C)
+    b = Budget(P, 16 * g.m)
+    with pytest.raises(P.SsspError) as e:
+        P.sssp_create(g.n, full.row_ptr, full.col, full.w, options=b.options, **csc)
+    assert e.value.code == P.SSSP_E_NOMEM and not b.live
