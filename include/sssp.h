@@ -172,7 +172,10 @@ typedef struct sssp_tuning {
                                 (0 = as many as fit)                                       */
     uint32_t tail_items;     /* rounds whose frontier and active set each make at most this
                                 many work items (32-vertex tiles and hub chunks) run in the
-                                16-CTA cluster kernel (0 = never)                          */
+                                16-CTA cluster kernel (0 = never).  A single query's
+                                label-setting or windowed rounds must also fit that kernel's
+                                shared memory: at most 12,288 vertices in either set, and at
+                                most max(16, 4096 / hub_degree) hub chunks                  */
 } sssp_tuning;
 
 /* The tuning a handle's solves use.  Errors: SSSP_E_INVAL. */
@@ -219,7 +222,8 @@ typedef struct sssp_tune_result {
 
 /* Autotuner: times single-source solves from `sources` (nsrc >= 1) on the
  * device for candidate tunings -- hub degree with chunk size, then the
- * cluster-tail work-item limit, then CTAs per SM, one parameter
+ * cluster-tail work-item limit (where two limits let the same rounds into the
+ * cluster kernel, one of them), then CTAs per SM, one parameter
  * group at a time starting from the handle's current tuning -- keeping the
  * fastest (best of `reps` passes, reps 0 = 3).  The winner is set on the
  * handle and put in the tuning cache under the graph's key.  Results of

@@ -110,6 +110,9 @@ __host__ __device__ __forceinline__ u32 light_prefix(const VDesc& x, u32 wtop, u
     return (u32)(((u64)b * x.deg + 254) / 255);
 }
 
+// Small-round kernel: most vertices in a round's frontier or active set.
+constexpr u32 kSmallEntries = 16 * 768;
+
 // Read-only description of one query's graph.
 struct InstDesc {
     const u64* out_off;     // CSR offsets, n + 1
@@ -222,7 +225,7 @@ struct RoundParams {
     u32 page_shift;
     u32 trace_cap;              // entries of `trace`
     u32 trace_base;             // round number of the first traced round
-    u32 tail_items;             // cluster tail kernel: most work items a round may have
+    u32 tail_items;             // cluster kernels: most work items a round may have
     u32 tail_chunks;            // small-round kernel: most hub chunks a list may have
     u32 small;                  // 1: single query whose ids fit 31 bits and edges 32 bits
                                 // (the small-round kernel's list entries)

@@ -33,6 +33,14 @@ TailKernel small_kernel(bool narrow, bool win);
 // n = 300 260 -> 127 us, n = 4096 602 -> 412 us, R-MAT 15 593 -> 497 us; degree 16, random
 // n = 20000 747 -> 540 us; half of it, 2048 edges, 602 us there.)
 inline u32 small_chunks(u32 hub_degree) { return std::max(16u, 4096u / hub_degree); }
+// The work items (32-entry tiles, hub chunks) that k_small's two limits add up to: a
+// larger tail_items lets no further round in.
+inline u32 small_items(u32 hub_degree) { return kSmallEntries / 32 + small_chunks(hub_degree); }
+// Whether two values of tail_items let the same rounds into k_small.
+inline bool same_small_rounds(u32 a, u32 b, u32 hub_degree) {
+    const u32 most = small_items(hub_degree);
+    return std::min(a, most) == std::min(b, most);
+}
 TailKernel tail_kernel(bool multi, bool narrow, const RoundParams& P);
 const void* barrier_selftest_fn();
 u32 tail_cluster_ctas();

@@ -37,6 +37,8 @@ constexpr u32 kSmallCTAs = kTailCTAs;
 constexpr u32 kSmallThreads = 512;
 constexpr u32 kSmallWarps = kSmallThreads / 32;
 constexpr u32 kSmallCap = 1024;      // entries of a CTA's active list, and of its frontier
+static_assert(kSmallEntries == kSmallCTAs * (kSmallCap * 3 / 4),
+              "a quarter of a list is left for the vertices that a round discovers");
 // Edges in flight per lane.  1: random n = 4096 and R-MAT tails 7-17% slower
 // (degrees above the group's lanes); 4: grids 7% slower (empty slots).
 constexpr u32 kSmallU = 2;
@@ -647,8 +649,7 @@ __device__ __forceinline__ void small_phase_bounds(const RoundParams& P, SmallSh
 // and few of them are hub chunks (P.tail_chunks).  Every CTA takes the same decision.
 __device__ __forceinline__ bool small_fits(const RoundParams& P, u32 items, u32 entries,
                                            u32 chunks) {
-    return items <= P.tail_items && entries <= kSmallCTAs * (kSmallCap * 3 / 4) &&
-           chunks <= P.tail_chunks;
+    return items <= P.tail_items && entries <= kSmallEntries && chunks <= P.tail_chunks;
 }
 
 template <class S, bool WIN>

@@ -176,9 +176,9 @@ bool same(const sssp_tuning& a, const sssp_tuning& b) {
 
 // Coordinate descent from `start`: each parameter group in turn, keeping a
 // candidate when it is at least 0.5% faster.  time(t, &ms) measures one
-// candidate.
+// candidate.  single_small: the rounds that fit run in k_small.
 template <class F>
-int sweep(const sssp_tuning& start, F time, sssp_tune_result* out) {
+int sweep(const sssp_tuning& start, bool single_small, F time, sssp_tune_result* out) {
     sssp_tuning best = start;
     double best_ms = 0;
     RC(time(best, &best_ms));
@@ -207,6 +207,7 @@ int sweep(const sssp_tuning& start, F time, sssp_tune_result* out) {
     for (u32 ti : kTailItems) {
         sssp_tuning t = g1;
         t.tail_items = ti;
+        if (single_small && same_small_rounds(ti, best.tail_items, best.hub_degree)) continue;
         RC(consider(t));
     }
     const sssp_tuning g2 = best;
@@ -405,7 +406,8 @@ int sssp_autotune(sssp_handle h, const uint32_t* sources, uint32_t nsrc, uint32_
         return SSSP_OK;
     };
     sssp_tune_result res{};
-    int rc = sweep(tuning_of(h), time, &res);
+    const RoundParams& P0 = h->single.P;
+    int rc = sweep(tuning_of(h), P0.small && !P0.pcnt && !P0.lc, time, &res);
     if (rc == SSSP_OK) rc = set_locked(h, res.best);
     cudaEventDestroy(e0);
     cudaEventDestroy(e1);
@@ -471,7 +473,7 @@ int sssp_autotune_batch(const sssp_handle* g, const uint32_t* sources, uint32_t 
         batch_key(g, k, key, sizeof(key));
         sssp_tuning cached{};
         if (tune_cache_find(key, &cached) == SSSP_OK) start = cached;
-        rc = sweep(start, time, &res);
+        rc = sweep(start, false, time, &res);
         if (rc == SSSP_OK) rc = sssp_tune_cache_put(key, &res.best);
     }
     if (st) cudaStreamSynchronize(st);
