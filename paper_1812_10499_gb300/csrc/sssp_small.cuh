@@ -326,9 +326,10 @@ __device__ __forceinline__ void small_relax(const RoundParams& P, SmallShared& s
         const u32 cta = (y * 0x9E3779B1u) >> 28;
         static_assert(kSmallCTAs == 16, "the owner is the hash's upper 4 bits");
         const u32 pos = dsm_add(map_cta(smem_u32(&s.nact[p]), cta), 1u);
-        // Its edges are read from the next phase on.
+        // Its edges are read from the next phase on.  (It has an in-edge; a vertex
+        // without out-edges may stand at the very end of the array.)
         prefetch_l2(P.g.in_adj + i0[i]);
-        prefetch_l2(P.g.out_adj + o0[i]);
+        if (od[i]) prefetch_l2(P.g.out_adj + o0[i]);
         ++a.pushed;
         if (id[i] > P.hub) a.chunks += (id[i] + P.chunk - 1) / P.chunk;
         if (pos < kSmallCap) {

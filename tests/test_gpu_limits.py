@@ -112,3 +112,19 @@ def test_graph_that_fits_without_descriptions(sssp_lib, loops, given_csc):
     with pytest.raises(P.SsspError) as e:
         P.sssp_create(g.n, full.row_ptr, full.col, full.w, options=b.options, **csc)
     assert e.value.code == P.SSSP_E_NOMEM and not b.live
+
+
+@LAYOUTS
+@pytest.mark.parametrize("mode,delta", [(oracle.RULE_THR, None), (oracle.RULE_THR, 9)],
+                         ids=["threshold", "windowed"])
+def test_last_vertex_without_out_edges(sssp_lib, layout, mode, delta):
+    """The adjacency fills its 2 MB exactly and the last vertices have no out-edge: their
+    rows begin at its end."""
+    n, sinks = 8192, 40
+    src = np.repeat(np.arange(n, dtype=np.uint32), 32)
+    col = (src + gg.uniform(3, 1, len(src), 1, n + sinks - 1).astype(np.uint32)) % np.uint32(n + sinks)
+    w = gg.uniform(3, 2, len(src), 1, 70).astype(np.uint32)
+    row_ptr = np.concatenate([np.arange(n + 1) * 32, np.full(sinks, 32 * n)]).astype(np.uint64)
+    g = gg.Graph(n + sinks, row_ptr, col, w)
+    assert 8 * g.m == 1 << 21
+    assert_parity(sssp_lib, g, 0, mode=mode, delta=delta, layout=layout)
