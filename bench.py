@@ -69,7 +69,7 @@ def window_delta(g, delta):
 #   per frontier vertex: 4 B list entry + 16 B offsets + 8 B own D + 8 B
 #     copy of its fixed lower bound;
 #   per in-edge scanned by k_cupdate: 8 B {source, w} + 16 B (D, C) of the
-#     source;
+#     source (counted for whole rows; the kernel reads the light prefix);
 #   per active vertex: 4 B list entry + 16 B offsets + 16 B own (D, C) +
 #     8 B new C + 4 B list append.
 B_OUT_EDGE, B_FRONT, B_IN_EDGE, B_ACTIVE = 16, 36, 24, 48
@@ -205,11 +205,12 @@ def _code_only(text):
 
 def kernel_source_sha256():
     """sha256 over the code (comments and layout ignored) of the round kernels'
-    sources and launch defaults: layout header, kernels, engine header with the
-    default hub and chunk sizes."""
+    sources and launch defaults: every kernel header, and the engine header
+    with the default hub and chunk sizes."""
     h = hashlib.sha256()
-    for f in ("sssp_dev.cuh", "sssp_round.cuh", "sssp_engine.h"):
-        text = open(os.path.join(ROOT, "paper_1812_10499_gb300", "csrc", f)).read()
+    csrc = os.path.join(ROOT, "paper_1812_10499_gb300", "csrc")
+    for f in sorted(x for x in os.listdir(csrc) if x.endswith(".cuh")) + ["sssp_engine.h"]:
+        text = open(os.path.join(csrc, f)).read()
         h.update(_code_only(text).encode())
     return h.hexdigest()
 
@@ -249,6 +250,34 @@ def alg_bytes(info):
     relax = B_OUT_EDGE * info["out_scanned"] + B_FRONT * info["front_visits"]
     cup = B_IN_EDGE * info["in_scanned"] + B_ACTIVE * info["active_visits"]
     return relax, cup
+
+
+def tail_kernel(rule):
+    """The cluster kernel that runs a single query's small rounds under a rule."""
+    return "k_tail" if RULES[rule] & (2 | 32) else "k_small"
+
+
+def kernel_table(prof, rule, peak):
+    """The round kernels of a profile (sssp_profile): launches, event time, share
+    and bytes.  k_relax reads every out-edge it counts, so its bytes over its time
+    are a rate.  k_cupdate counts every in-edge of a scanned vertex, also those too
+    heavy to matter, which it does not read: its bytes are those of a scan
+    of whole rows, and the rate is an equivalent one, without a fraction of the peak."""
+    gc, tc = prof["grid_counters"], prof["tail_counters"]
+    rows = [("k_cupdate", alg_bytes(gc)[1], prof["cupdate_ms"], prof["cupdate_launches"], True),
+            ("k_relax", alg_bytes(gc)[0], prof["relax_ms"], prof["relax_launches"], False),
+            (tail_kernel(rule), sum(alg_bytes(tc)), prof["tail_ms"], prof["tail_launches"], False)]
+    out = {}
+    for k, b, t_ms, n, equivalent in rows:
+        if n == 0 or t_ms <= 0:
+            continue
+        gbs = b / (t_ms * 1e-3) / 1e9
+        rate = {"equivalent_gbs": gbs} if equivalent else {"achieved_gbs": gbs, "frac": gbs / peak}
+        out[k] = {"launches": n, "ms": t_ms, "bytes": b, **rate}
+    total = sum(v["ms"] for v in out.values())
+    for v in out.values():
+        v["share"] = v["ms"] / total
+    return out
 
 
 def reduce_over_ranks(dist, device, local_ms, local_units):
@@ -482,7 +511,7 @@ def run_ours(args):
     ms, edges = reduce_over_ranks(dist, "cuda", ms, args.steps * m_reach)
     value = edges / (ms * 1e-3) / 1e9
     # Kernels launched per solve, counted by the library (start, round kernels
-    # including the cluster tail kernel of every device-loop iteration, output).
+    # including the cluster kernel of every device-loop iteration, output).
     launches = args.steps * sum(i["kernel_launches"] for i in infos)
 
     # ---- roofline: every kernel's launches timed with CUDA events on the
@@ -505,24 +534,7 @@ def run_ours(args):
     P.sssp_solve_ex(h, sources[0], dist=False, stream=stream)
     per_iter = P.sssp_profile_rounds(h)
     P.sssp_profile(h, False)
-    gc, tc = prof["grid_counters"], prof["tail_counters"]
-    kern = {
-        "k_cupdate": (B_IN_EDGE * gc["in_scanned"] + B_ACTIVE * gc["active_visits"],
-                      prof["cupdate_ms"], prof["cupdate_launches"]),
-        "k_relax": (B_OUT_EDGE * gc["out_scanned"] + B_FRONT * gc["front_visits"],
-                    prof["relax_ms"], prof["relax_launches"]),
-        "k_tail": (alg_bytes(tc)[0] + alg_bytes(tc)[1], prof["tail_ms"], prof["tail_launches"]),
-    }
-    kernels = {}
-    for k, (b, t_ms, n) in kern.items():
-        if n == 0 or t_ms <= 0:
-            continue
-        kernels[k] = {"launches": n, "ms": t_ms, "bytes": b,
-                      "achieved_gbs": b / (t_ms * 1e-3) / 1e9,
-                      "frac": b / (t_ms * 1e-3) / 1e9 / peak, "share": 0.0}
-    tot_ms = sum(v["ms"] for v in kernels.values())
-    for v in kernels.values():
-        v["share"] = v["ms"] / tot_ms
+    kernels = kernel_table(prof, args.rule, peak)
     if args.loop == "persistent":
         # One launch of k_solve per solve: events around each solve call.
         pairs = []
@@ -542,17 +554,23 @@ def run_ours(args):
                   "four small start/output kernels)")
     else:
         kernel = max(kernels, key=lambda k: kernels[k]["ms"])      # the dominant kernel
-        b, t_ms, n = kern[kernel]
-        ms_per_launch = t_ms / n
-        bytes_per_launch = b / n
+        ms_per_launch = kernels[kernel]["ms"] / kernels[kernel]["launches"]
+        bytes_per_launch = kernels[kernel]["bytes"] / kernels[kernel]["launches"]
         timing = ("CUDA events around every launch on the solve stream; the host launches the "
-                  "device loop's iterations (k_relax, k_cupdate, cluster tail kernel k_tail) as "
-                  "the timed solves run them; algorithmic bytes from the work counters of the "
-                  "rounds each kernel ran, with every in-edge of a scanned vertex counted, also "
-                  "those too heavy to matter, which k_cupdate does not read")
-    dom_gbs = bytes_per_launch / (ms_per_launch * 1e-3) / 1e9
+                  f"device loop's iterations (k_relax, k_cupdate, cluster kernel "
+                  f"{tail_kernel(args.rule)}) as the timed solves run them; bytes from the work "
+                  "counters of the rounds each kernel ran")
+    # The roofline figure: bytes that the kernel moves over its time.  Where the
+    # counters give whole rows of in-edges (k_cupdate, k_solve), the DRAM traffic that
+    # ncu measured stands in, if the record is of these kernels; else none is given.
+    whole_rows = kernel in ("k_cupdate", "k_solve")
+    counted_gbs = bytes_per_launch / (ms_per_launch * 1e-3) / 1e9
     traffic, traffic_src = measured_traffic(kernel, args.config, bytes_per_launch)
-    # Whole step: all algorithmic bytes of the 8 solves over the timed step.
+    if not whole_rows:
+        dom_gbs = counted_gbs
+    else:
+        dom_gbs = traffic / (ms_per_launch * 1e-3) / 1e9 if traffic else None
+    # Whole step: the counted bytes of the 8 solves over the timed step.
     step_gbs = step_bytes / (ms_local / args.steps * 1e-3) / 1e9
 
     # ---- end to end through the public host API (dist copied to host)
@@ -592,15 +610,20 @@ def run_ours(args):
                    "l2": "inputs larger than L2 (CSR+CSC+state > 1 GB)",
                    "parallelism": f"replicas x{ws}"},
         "roofline": {"bound": "hbm", "kernel": kernel, "achieved": dom_gbs, "peak": peak,
-                     "peak_kind": peak_kind, "unit": "GB/s", "frac": dom_gbs / peak,
+                     "peak_kind": peak_kind, "unit": "GB/s",
+                     "frac": dom_gbs / peak if dom_gbs is not None else None,
+                     "achieved_is": ("DRAM traffic measured by ncu over the kernel's time"
+                                     if whole_rows else "bytes counted over the kernel's time"),
+                     **({"equivalent_gbs": counted_gbs} if whole_rows else {}),
                      "traffic": traffic, "traffic_source": traffic_src,
                      "bytes_per_launch": bytes_per_launch,
                      "ms_per_launch": ms_per_launch, "timing": timing,
                      "kernels": kernels,
                      "step": {"bytes": step_bytes, "ms": ms_local / args.steps,
-                              "achieved": step_gbs, "frac": step_gbs / peak,
-                              "what": "algorithmic bytes of all kernels of the 8 solves over "
-                                      "the timed step (device loop, no profiling)"},
+                              "equivalent_gbs": step_gbs,
+                              "what": "counted bytes of all kernels of the 8 solves (whole rows "
+                                      "of in-edges, most of which are not read) over the timed "
+                                      "step (device loop, no profiling)"},
                      "per_iteration_first_source": {
                          "relax_ms": [round(float(x), 4) for x in per_iter[0]],
                          "cupdate_ms": [round(float(x), 4) for x in per_iter[1]],
