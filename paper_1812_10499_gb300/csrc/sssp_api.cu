@@ -419,9 +419,12 @@ int alloc_lists(Context& c, u64 capS, u64 capH, u64 capC) {
 // one of kHotSlots candidate slots, kHotStride bytes apart, of one allocation:
 // the slot that the tail kernel's cluster reaches with the shortest chain of
 // atomics (k_place_probe).  Which slot that is depends on where the
-// allocation lands in physical memory, and the latency-bound rounds -- each
-// a chain of waits on these words -- differ by up to 14% between a good slot
-// and a bad one.  SSSP_HOT_SLOT=<i> forces slot i (for measurements).
+// allocation lands in physical memory, and the latency-bound rounds of k_tail
+// -- each a chain of waits on these words -- differ by up to 14% between a good
+// slot and a bad one.  (k_small reads them at its start and end only.)  The
+// scalars of up to 36 queries fit beside the block: batches of 36, 40, 56, 60 and 64
+// small graphs gain alike over the kernels before the block's words were spread out
+// (1.24 to 1.29 times).  SSSP_HOT_SLOT=<i> forces slot i (for measurements).
 int alloc_hot(Context& c, u32 nivar, cudaStream_t st) {
     constexpr u32 kHotSlots = 16, kHotStride = 4096;
     const size_t bytes = (size_t)kHotSlots * kHotStride;

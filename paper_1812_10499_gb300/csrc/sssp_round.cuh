@@ -39,7 +39,6 @@ namespace sssp {
 
 constexpr u32 kFull = 0xFFFFFFFFu;
 constexpr u32 kWarps = 8;       // warps per CTA (256 threads)
-constexpr u32 kSmallGrid = 32;  // grids up to this many CTAs run latency-bound rounds
 constexpr u32 kQFlush = 96;     // entries a warp append buffer hands over per atomic
 constexpr u32 kQCap = kQFlush + 32;
 // Build-time tuning: CTAs per SM the round kernels are compiled for, and
@@ -1143,13 +1142,14 @@ __device__ __forceinline__ u64 decide(const RoundParams& P, u64 dy, u64 cy, u64 
     return fix ? dy : cn;
 }
 
-// SHATOM (the cluster tail kernel): with the compact layout each edge's
-// 32-bit term goes into its owner's slot by a shared-memory atomicMin
-// instead of the segmented scan -- fewer dependent instructions per batch,
-// which is what the small rounds wait on (random n = 4096 -15%, R-MAT 22
-// +3%).  In large rounds, where many lanes share an owner, the scan is
-// faster, and with the wide layout's 64-bit terms the atomics cost 1.4% on
-// the 4096^2 grid, so both keep the scan.
+// SHATOM (k_tail): with the compact layout each edge's 32-bit term goes into
+// its owner's slot by a shared-memory atomicMin instead of the segmented scan
+// -- fewer dependent instructions per batch, which is what the small rounds
+// wait on.  In large rounds, where many lanes share an owner, the scan is
+// faster, and with the wide layout's 64-bit terms the atomics lost a little
+// (+1.4%), so both keep the scan.  (Measured while k_tail ran every small round,
+// random n = 4096 -15%; it now runs those of batches, predecessor counts and
+// label-correcting rounds.)
 template <bool MULTI, class L, bool SHATOM = false>
 __device__ void cup_small(const RoundParams& P, InstCache<typename L::Term>* ic, WarpStage<typename L::CSlot>& st, u32 t, u32 ts,
                           u32 nas, u32 r, u32 cur, u32 lane, u64* smin, u64 thr0, u64 minD0,

@@ -66,6 +66,10 @@ struct __align__(16) SmallSlot {
     u32 flags, pad[3];               // 1: a list overflowed, 2: the target is fixed
 };
 
+// The CTA's counts that a decided vertex adds to: entries of the two active lists,
+// frontier entries, those that relax, those fixed.
+enum : u32 { kActive0 = 0, kActive1 = 1, kFront = 2, kLive = 3, kNewFixed = 4, kCounts = 5 };
+
 struct SmallShared {
     ActEntry act[2][kSmallCap];
     FrontEntry fr[kSmallCap];
@@ -75,16 +79,12 @@ struct SmallShared {
     u32 wpush[kSmallWarps], wchunk[kSmallWarps];   // ... and discoveries
     u64 bigmin;
     u32 big[kBigCap];                // entries for the whole CTA
-    u32 nact[2];                     // entries of the lists
-    u32 nfr, live, nfix;             // frontier entries; those that relax; those fixed
+    u32 cnt[kCounts];
     u32 nbig, chunks, fchunks, flags;
 };
 
 // --------------------------------------------------- distributed shared memory
 
-__device__ __forceinline__ u32 smem_u32(const void* p) {
-    return (u32)__cvta_generic_to_shared(p);
-}
 __device__ __forceinline__ u32 map_cta(u32 addr, u32 cta) {
     u32 r;
     asm volatile("mapa.shared::cluster.u32 %0, %1, %2;\n" : "=r"(r) : "r"(addr), "r"(cta));
@@ -114,14 +114,6 @@ __device__ __forceinline__ void small_sync() {
 }
 
 // ------------------------------------------------------------------ layouts
-
-// Warp minimum, to every lane: the upper halves, then the lower halves of the
-// lanes that hold the least upper half.
-__device__ __forceinline__ u64 warp_least(u64 v) {
-    const u32 hi = __reduce_min_sync(kFull, (u32)(v >> 32));
-    const u32 lo = __reduce_min_sync(kFull, (u32)(v >> 32) == hi ? (u32)v : kFull);
-    return ((u64)hi << 32) | lo;
-}
 
 // State access of the two layouts.  Records, filter words and change marks are
 // written by other CTAs during the kernel, so they are read from L2.
@@ -158,7 +150,7 @@ struct SmallWide {
     __device__ static Dist fixed_dist(const Rec* p, u32 cur) {
         return __ldcg(&p->cf[cur]) & kCMask;
     }
-    __device__ static Dist wmin(Dist v) { return warp_least(v); }
+    __device__ static Dist wmin(Dist v) { return warp_min64(v); }
     // A relaxation target: open (not fixed), its packed D, outWeight, in-degree.
     struct Tgt {
         u64 d, c;
@@ -325,7 +317,7 @@ __device__ __forceinline__ void small_relax(const RoundParams& P, SmallShared& s
         const u32 y = e[i].x;
         const u32 cta = (y * 0x9E3779B1u) >> 28;
         static_assert(kSmallCTAs == 16, "the owner is the hash's upper 4 bits");
-        const u32 pos = dsm_add(map_cta(smem_u32(&s.nact[p]), cta), 1u);
+        const u32 pos = dsm_add(map_cta(smem_addr(&s.cnt[p]), cta), 1u);
         // Its edges are read from the next phase on.  (It has an in-edge; a vertex
         // without out-edges may stand at the very end of the array.)
         prefetch_l2(P.g.in_adj + i0[i]);
@@ -333,7 +325,7 @@ __device__ __forceinline__ void small_relax(const RoundParams& P, SmallShared& s
         ++a.pushed;
         if (id[i] > P.hub) a.chunks += (id[i] + P.chunk - 1) / P.chunk;
         if (pos < kSmallCap) {
-            const u32 at = map_cta(smem_u32(&s.act[p][pos]), cta);
+            const u32 at = map_cta(smem_addr(&s.act[p][pos]), cta);
             dsm_st4(at, y, id[i], (u32)i0[i], (u32)(i0[i] >> 32));
             dsm_st4(at + 16, (u32)o0[i], (u32)(o0[i] >> 32), od[i], ow[i]);
         } else {
@@ -366,7 +358,7 @@ __device__ __forceinline__ void small_phase_relax(const RoundParams& P, SmallSha
                                                   u32 cur, u32 lane, u32 wib, SmallAcc<S>& a) {
     typedef typename S::Dist Dist;
     constexpr u32 U = kSmallU;
-    const u32 n = s.nfr;
+    const u32 n = s.cnt[kFront];
     const u32 gs = group_shift(n), sub = lane & ((1u << gs) - 1u);
     const u32 lim = max(kGroupDeg, (4 * U) << gs);
     typename S::Rec* rec = S::rec(P);
@@ -498,12 +490,12 @@ __device__ __forceinline__ void small_decide(const RoundParams& P, SmallShared& 
     const u32 ms = __ballot_sync(kFull, sv), mf = __ballot_sync(kFull, fl);
     const u32 mx = WIN ? __ballot_sync(kFull, fx) : mf;
     const u32 mfix = WIN ? __ballot_sync(kFull, fix) : mf;
-    // Lanes 0 to 3 reserve the places and count, side by side (the words
-    // nact[0], nact[1], nfr, live, nfix are consecutive).
+    // Lanes 0 to 3 reserve the places and count, side by side.
     u32 got = 0;
+    static_assert(kFront == 2 && kLive == 3 && kNewFixed == 4, "of lanes 1 to 3");
     {
         const u32 cnt = __popc(lane == 0 ? ms : lane == 1 ? mf : lane == 2 ? mx : mfix);
-        if (lane < 4 && cnt) got = atomicAdd(&s.nact[lane == 0 ? q : lane + 1], cnt);
+        if (lane < 4 && cnt) got = atomicAdd(&s.cnt[lane == 0 ? q : lane + 1], cnt);
     }
     const u32 bs = __shfl_sync(kFull, got, 0), bf = __shfl_sync(kFull, got, 1);
     if (sv) {
@@ -533,7 +525,7 @@ __device__ __forceinline__ void small_phase_bounds(const RoundParams& P, SmallSh
     typedef typename S::Dist Dist;
     constexpr u32 U = kSmallU;
     const u32 cur = r & 1u;
-    const u32 n = s.nact[p];
+    const u32 n = s.cnt[p];
     const u32 gs = group_shift(n), sub = lane & ((1u << gs) - 1u);
     const u32 lim = max(kGroupDeg, (4 * U) << gs);
     const typename S::Rec* rec = S::rec(P);
@@ -685,10 +677,10 @@ __global__ void __launch_bounds__(kSmallThreads, 1)
 
     // The lists, dealt round-robin over the CTAs.
     if (tid == 0) {
-        s.nbig = s.chunks = s.fchunks = s.nfix = s.flags = 0;
-        s.nact[0] = (nas + nah + kSmallCTAs - 1 - rank) / kSmallCTAs;
-        s.nact[1] = 0;
-        s.nfr = s.live = (nfs + nfh + kSmallCTAs - 1 - rank) / kSmallCTAs;
+        s.nbig = s.chunks = s.fchunks = s.flags = s.cnt[kNewFixed] = 0;
+        s.cnt[0] = (nas + nah + kSmallCTAs - 1 - rank) / kSmallCTAs;
+        s.cnt[1] = 0;
+        s.cnt[kFront] = s.cnt[kLive] = (nfs + nfh + kSmallCTAs - 1 - rank) / kSmallCTAs;
     }
     for (u32 i = tid; rank + kSmallCTAs * i < nfs + nfh; i += kSmallThreads) {
         const u32 k = rank + kSmallCTAs * i;
@@ -741,7 +733,7 @@ __global__ void __launch_bounds__(kSmallThreads, 1)
     for (;;) {
         const u32 cur = r & 1u;
         // Step (a) of round r, then the minima over the active set.
-        if (tid == 0) s.nact[p ^ 1u] = 0;
+        if (tid == 0) s.cnt[p ^ 1u] = 0;
         small_phase_relax<S, WIN>(P, s, p, cur, lane, wib, a);
         {
             const Dist d = S::wmin(a.fd), t = S::wmin(a.ft);
@@ -759,20 +751,21 @@ __global__ void __launch_bounds__(kSmallThreads, 1)
         __syncthreads();
         if (wib == 0) {
             const bool in = lane < kSmallWarps;
-            const u64 d = warp_least(in ? s.wd[lane] : kInf64);
-            const u64 t = warp_least(in ? s.wt[lane] : kInf64);
+            const u64 d = warp_min64(in ? s.wd[lane] : kInf64);
+            const u64 t = warp_min64(in ? s.wt[lane] : kInf64);
             const u32 np = __reduce_add_sync(kFull, in ? s.wpush[lane] : 0u);
             const u32 nc = __reduce_add_sync(kFull, in ? s.wchunk[lane] : 0u);
             const u32 flags = s.flags;
             if (lane < kSmallCTAs) {
-                const u32 at = map_cta(smem_u32(&s.xb[rank]), lane);
+                const u32 at = map_cta(smem_addr(&s.xb[rank]), lane);
                 dsm_st4(at, (u32)d, (u32)(d >> 32), (u32)t, (u32)(t >> 32));
                 dsm_st4(at + 16, 0u, np, nc, 0u);
                 dsm_st4(at + 32, flags, 0u, 0u, 0u);
             }
         } else if (wib == 1 && lane == 0) {
-            a.front += s.live;
-            s.chunks = s.fchunks = s.nbig = s.nfr = s.nfix = s.live = 0;
+            a.front += s.cnt[kLive];
+            s.chunks = s.fchunks = s.nbig = 0;
+            s.cnt[kFront] = s.cnt[kLive] = s.cnt[kNewFixed] = 0;
         }
         small_sync();
         u32 nact = surv, chunks = schunks;
@@ -793,10 +786,10 @@ __global__ void __launch_bounds__(kSmallThreads, 1)
         small_phase_bounds<S, WIN>(P, s, p, r, thr, minD, target, lane, wib, a);
         __syncthreads();
         if (wib == 0) {
-            const u32 ns = s.nact[p ^ 1u], nl = s.live, nf = s.nfix, ch = s.chunks,
+            const u32 ns = s.cnt[p ^ 1u], nl = s.cnt[kLive], nf = s.cnt[kNewFixed], ch = s.chunks,
                       fch = s.fchunks, flags = s.flags;
             if (lane < kSmallCTAs) {
-                const u32 at = map_cta(smem_u32(&s.xa[rank]), lane);
+                const u32 at = map_cta(smem_addr(&s.xa[rank]), lane);
                 dsm_st4(at, fch, 0u, 0u, 0u);
                 dsm_st4(at + 16, nl, ns, ch, nf);
                 dsm_st4(at + 32, flags, 0u, 0u, 0u);
@@ -829,7 +822,7 @@ __global__ void __launch_bounds__(kSmallThreads, 1)
     // the survivors' folds.  (r already counts the next round there.)
     const u32 cu = r & 1u;
     if (end_status == kRunning && !err_rounds) {
-        const u32 n = s.nact[p] < kSmallCap ? s.nact[p] : kSmallCap;
+        const u32 n = s.cnt[p] < kSmallCap ? s.cnt[p] : kSmallCap;
         for (u32 i = tid; i < n; i += kSmallThreads) {
             const ActEntry en = s.act[p][i];
             if (en.deg > P.hub)
@@ -838,7 +831,7 @@ __global__ void __launch_bounds__(kSmallThreads, 1)
                 put_small(P, P.L.AS[cu], atomicAdd(&ctl->nAS[cu], 1u), en.g);
         }
         if (!cup_only) {
-            for (u32 i = tid; i < s.nfr; i += kSmallThreads) {
+            for (u32 i = tid; i < s.cnt[kFront]; i += kSmallThreads) {
                 const FrontEntry f = s.fr[i];
                 const u32 g = f.g & ~kFixedEntry;
                 if (f.g & kFixedEntry) S::set_c(rec + g, cu ^ 1u, (Dist)s.fdist[i], true);

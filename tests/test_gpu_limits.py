@@ -1,4 +1,5 @@
-"""Limits that the sizes of a call cross: hub chunks in the cluster kernel's rounds."""
+"""Limits that the sizes of a call cross: hub chunks in the cluster kernel's rounds,
+device memory, queries of a batch, the end of the adjacency."""
 import numpy as np
 import pytest
 
@@ -128,3 +129,28 @@ def test_last_vertex_without_out_edges(sssp_lib, layout, mode, delta):
     g = gg.Graph(n + sinks, row_ptr, col, w)
     assert 8 * g.m == 1 << 21
     assert_parity(sssp_lib, g, 0, mode=mode, delta=delta, layout=layout)
+
+
+@LAYOUTS
+@pytest.mark.parametrize("mode,delta", [(oracle.RULE_THR, None), (oracle.LABEL_CORRECT, None),
+                                        (oracle.RULE_THR, 15)],
+                         ids=["threshold", "correcting", "windowed"])
+def test_more_queries_than_a_cta_keeps_minima_of(sssp_lib, layout, mode, delta):
+    """1100 queries of one batch: the minima and counts of those after the 1024th go to
+    global memory one by one.  Every query's distances and rounds are its own run's."""
+    P, n, k = sssp_lib, 170, 1100
+    g = gg.random_var_graph(n, 1, 7, 1, 40, 12)
+    opt = P.sssp_options_default()
+    opt.layout, opt.rule = layout, mode
+    if delta is not None:
+        opt.rule, opt.delta = P.SSSP_RULE_WINDOWED, delta
+    refs = [oracle.round_r(g, s, mode=mode, delta=delta) for s in range(n)]
+    sources = [(7 * i) % n for i in range(k)]
+    h = P.sssp_create(g.n, g.row_ptr, g.col, g.w, options=opt)
+    try:
+        dist, rounds = P.sssp_solve_batch([h] * k, sources)
+    finally:
+        P.sssp_destroy(h)
+    for i, s in enumerate(sources):
+        assert rounds[i] == refs[s].rounds, i
+        assert np.array_equal(dist[i], refs[s].dist), i
