@@ -130,9 +130,11 @@ typedef struct sssp_graph* sssp_handle;
 typedef struct sssp_server sssp_server;
 
 /* Device-memory allocator hook.  alloc returns a device pointer aligned to at
- * least 256 bytes or NULL; free releases it.  Both are called only from
- * sssp_create / sssp_destroy / sssp_serve_open / sssp_serve_close.  NULL
- * hooks mean cudaMalloc / cudaFree. */
+ * least 256 bytes or NULL; free releases it.  Both are called from
+ * sssp_create / sssp_destroy, the calls that set or search a tuning,
+ * sssp_serve_open / sssp_serve_close, and from solves that need more than the
+ * handle holds: a batch (its workspace, kept for the next one) and lower
+ * bounds to the host.  NULL hooks mean cudaMalloc / cudaFree. */
 typedef void* (*sssp_alloc_fn)(size_t bytes, void* ctx);
 typedef void (*sssp_free_fn)(void* ptr, void* ctx);
 

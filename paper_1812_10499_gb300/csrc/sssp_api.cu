@@ -176,9 +176,9 @@ int build_loop(Context& c) {
 }
 
 // A profiled solve in the device loop's schedule: each iteration launches
-// k_relax, k_cupdate and the cluster tail kernel from the host, with events
-// around each launch, and snapshots of the control block after k_cupdate and
-// after k_tail that split the work counters by the kernel that did the work.
+// k_relax, k_cupdate and the small rounds' cluster kernel from the host, with events
+// around each launch, and snapshots of the control block after k_cupdate and after
+// the cluster kernel, which split the work counters by the kernel that did the work.
 int profile_graph_schedule(Context& c, cudaStream_t st) {
     const void* fr = relax_fn(c.multi, c.narrow, c.P.pcnt != nullptr);
     const void* fc = cupdate_fn(c.multi, c.narrow, c.P.pcnt != nullptr);
@@ -194,7 +194,7 @@ int profile_graph_schedule(Context& c, cudaStream_t st) {
     }
     if (!c.h_snap) CK(cudaHostAlloc((void**)&c.h_snap, 2 * sizeof(Ctl), cudaHostAllocDefault));
     // Launch attributes as in the device loop: the records' L2 window on
-    // every kernel, the cluster shape on the tail kernel.
+    // every kernel, the cluster shape on the third.
     cudaLaunchAttribute at[2];
     at[0].id = cudaLaunchAttributeAccessPolicyWindow;
     at[0].val.accessPolicyWindow = c.l2win;
